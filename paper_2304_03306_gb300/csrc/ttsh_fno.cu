@@ -856,20 +856,6 @@ __global__ void __launch_bounds__(256) modemix_bwd_kernel(const float* __restric
   }
 }
 
-// Adam with bias correction on the FP32 master weights
-__global__ void adam_kernel(float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  th[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
@@ -909,7 +895,70 @@ __global__ void to_double_scaled_kernel(const float* __restrict__ src, long long
   if (p < n) dst[p] = (double)src[p] * (double)scale;
 }
 
+// Adam with bias correction on the FP32 master weights and the BF16 copies of the mixing weights in the same pass: parameter i
+// of a layer's segment (Wr | Wi | W | b, `lay` long, the first `msz2` values spectral) has its
+// copy at the same place of that layer's BF16 segment (Wr | Wi | W^T | W).
+__global__ void __launch_bounds__(256) adam_bf16_kernel(float4* __restrict__ th, const float4* __restrict__ g,
+                                                        float4* __restrict__ m, float4* __restrict__ v, long long n,
+                                                        float lr, float b1, float b2, float eps, float c1, float c2,
+                                                        long long first, long long lay, long long msz2, int L,
+                                                        long long blay, __nv_bfloat16* __restrict__ wbf) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long i = 4 * q;
+  if (i >= n) return;
+  const bool whole = i + 4 <= n;
+  float t4[4], g4[4], m4[4], v4[4];
+  if (whole) {
+    *reinterpret_cast<float4*>(t4) = th[q];
+    *reinterpret_cast<float4*>(g4) = g[q];
+    *reinterpret_cast<float4*>(m4) = m[q];
+    *reinterpret_cast<float4*>(v4) = v[q];
+  } else {
+    for (int k = 0; k < 4; ++k) {
+      const bool in = i + k < n;
+      t4[k] = in ? reinterpret_cast<const float*>(th)[i + k] : 0.f;
+      g4[k] = in ? reinterpret_cast<const float*>(g)[i + k] : 0.f;
+      m4[k] = in ? reinterpret_cast<const float*>(m)[i + k] : 0.f;
+      v4[k] = in ? reinterpret_cast<const float*>(v)[i + k] : 0.f;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float gi = g4[k];
+    const float mi = b1 * m4[k] + (1.f - b1) * gi;
+    const float vi = b2 * v4[k] + (1.f - b2) * gi * gi;
+    m4[k] = mi;
+    v4[k] = vi;
+    t4[k] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  }
+  if (whole) {
+    th[q] = *reinterpret_cast<const float4*>(t4);
+    m[q] = *reinterpret_cast<const float4*>(m4);
+    v[q] = *reinterpret_cast<const float4*>(v4);
+  } else {
+    for (int k = 0; k < 4 && i + k < n; ++k) {
+      reinterpret_cast<float*>(th)[i + k] = t4[k];
+      reinterpret_cast<float*>(m)[i + k] = m4[k];
+      reinterpret_cast<float*>(v)[i + k] = v4[k];
+    }
+  }
+  const long long l = (i - first) / lay, r = i - first - l * lay;
+  if (i < first || l >= L || r >= msz2 + CW * CW) return;
+  __nv_bfloat16* seg = wbf + l * blay;
+  __nv_bfloat162 e[2] = {__floats2bfloat162_rn(t4[0], t4[1]), __floats2bfloat162_rn(t4[2], t4[3])};
+  if (r < msz2) {
+    *reinterpret_cast<uint2*>(seg + r) = *reinterpret_cast<const uint2*>(e);
+  } else {
+    const int k = (int)(r - msz2);   // W[i][o], o fastest: W^T first, then W
+    *reinterpret_cast<uint2*>(seg + msz2 + CW * CW + k) = *reinterpret_cast<const uint2*>(e);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) seg[msz2 + ((k % CW) + o) * CW + k / CW] = reinterpret_cast<const __nv_bfloat16*>(e)[o];
+  }
+}
+
 }  // namespace fno_dev
+
+#include "ttsh_fno_fused.cuh"
 
 // =======================================================================================
 // Host side
@@ -947,6 +996,10 @@ struct ttsh_fno {
   // n <= 512, 2m <= 32): Fx [32][n], Bx [n][32], Fx^T [n][32], Bx^T [32][n], zero-padded
   __nv_bfloat16 *FxB = nullptr, *BxB = nullptr, *FxTB = nullptr, *BxTB = nullptr;
   bool tc_rows = false;
+  // two kernels a layer (ttsh_fno_fused.cuh): tc_rows, fused_columns and n <= 512
+  bool fused = false;
+  int cluster = 8;              // blocks per cluster of the column kernels
+  double* loss = nullptr;       // in the same 64 bytes as tc_err, behind it
   long long adam_t = 0;
   std::vector<void*> allocs;
 };
@@ -1039,8 +1092,233 @@ cudaError_t refresh_bf16(ttsh_fno* f) {
   return cudaGetLastError();
 }
 
+// ---- two kernels a layer ----
+// Launch, optionally as a programmatic dependent launch (the kernel stages what no kernel of this
+// pass writes while the previous one still runs; never the first kernel of a pass, so that the
+// weights it stages early were complete before the pass began) and in clusters of `cl` blocks.
+template <typename A>
+cudaError_t launch_layer(void (*k)(A), dim3 grid, int block, int smem, cudaStream_t s, bool pdl, int cl, const A& a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (pdl) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cl > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)cl;
+    at[na].val.clusterDim.y = 1;
+    at[na++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = (unsigned)na;
+  return cudaLaunchKernelEx(&cfg, k, a);
+}
+
+template <int MODE, int T, bool TRAIN>
+cudaError_t row_one(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup) {
+  const int smem = row_smem(MODE, TRAIN, f->n);
+  auto k = &row_layer_kernel<MODE, T, TRAIN>;
+  if (setup) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // resident blocks per SM: tensor memory (64 T of 512 columns each), shared memory, 64 warps
+  int per = 8 / T;
+  const int fit = (227 * 1024) / (smem + 2048);
+  if (fit < per) per = fit < 1 ? 1 : fit;
+  if (per > 16 / T / 2) per = 16 / T / 2;
+  const long long cap = 152LL * per;
+  return launch_layer(k, dim3((unsigned)(a.Q < cap ? a.Q : cap)), 128 * T, smem, f->stream, pdl, 1, a);
+}
+
+template <int MODE, bool TRAIN>
+cudaError_t run_row(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup = false) {
+  if (f->n <= 128) return row_one<MODE, 1, TRAIN>(f, a, pdl, setup);
+  if (f->n == 256) return row_one<MODE, 2, TRAIN>(f, a, pdl, setup);
+  return row_one<MODE, 4, TRAIN>(f, a, pdl, setup);
+}
+
+template <bool ADJ>
+cudaError_t run_column(ttsh_fno* f, const ColArgs& a, int B, bool pdl, bool setup = false) {
+  const int cs = f->cluster, smem = col_smem(f->n, 2 * f->m, cs);
+  auto k = cs == 8 ? &column_layer_kernel<8, ADJ> : &column_layer_kernel<4, ADJ>;
+  if (setup) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return launch_layer(k, dim3((unsigned)(cs * f->m), (unsigned)B), kColThreads, smem, f->stream, pdl, cs, a);
+}
+
+cudaError_t fused_setup(ttsh_fno* f) {
+  const RowArgs r{};
+  const ColArgs c{};
+  cudaError_t e = run_row<R_LIFT, false>(f, r, false, true);
+  if (e == cudaSuccess) e = run_row<R_FWD, false>(f, r, false, true);
+  if (e == cudaSuccess) e = run_row<R_FWD, true>(f, r, false, true);
+  if (e == cudaSuccess) e = run_row<R_LAST, false>(f, r, false, true);
+  if (e == cudaSuccess) e = run_row<R_LAST_TRAIN, true>(f, r, false, true);
+  if (e == cudaSuccess) e = run_row<R_BWD, true>(f, r, false, true);
+  if (e == cudaSuccess) e = run_row<R_BWD_FIRST, true>(f, r, false, true);
+  if (e == cudaSuccess) e = run_column<false>(f, c, 1, false, true);
+  if (e == cudaSuccess) e = run_column<true>(f, c, 1, false, true);
+  auto wg = [&](auto k) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+  };
+  wg(&wgrad_kernel<WA_RAW, WD_ONE>);
+  wg(&wgrad_kernel<WA_GELU, WD_OUTER>);
+  wg(&wgrad_kernel<WA_GELU, WD_RAW>);
+  wg(&wgrad_kernel<WA_LIFT, WD_OUTER>);
+  wg(&wgrad_kernel<WA_LIFT, WD_RAW>);
+  wg(&wgrad_kernel<WA_X, WD_RAW>);
+  return e;
+}
+
+RowArgs row_args(ttsh_fno* f, int B) {
+  RowArgs a{};
+  a.n = f->n;
+  a.J = 2 * f->m;
+  a.Q = (long long)B * f->n;
+  a.P = (long long)B * f->nn;
+  a.err = f->tc_err;
+  a.X = f->Hx;
+  a.Z = f->Z;
+  return a;
+}
+
+ColArgs column_args(ttsh_fno* f, int l) {
+  ColArgs c{};
+  c.X = f->Hx;
+  c.Z = f->Z;
+  c.Gr = f->Gr;
+  c.Gi = f->Gi;
+  c.Wr = f->wbf + f->boff_Wr[l];
+  c.Wi = f->wbf + f->boff_Wi[l];
+  c.n = f->n;
+  c.m = f->m;
+  c.err = f->tc_err;
+  return c;
+}
+
+// Forward pass; with a target it also leaves the loss in f->loss, the last layer's dz (BF16) and
+// its row transform, from which backward_fused starts.
+ttsh_status forward_fused(ttsh_fno* f, const float* x, int B, float* out, const float* target) {
+  const int L = f->L;
+  RowArgs a = row_args(f, B);
+  a.x = x;
+  a.Wp = f->theta + f->off_Wp;
+  a.bp = f->theta + f->off_bp;
+  a.C = f->FxB;
+  a.hb = f->hb[0];
+  FNO_CUDA((run_row<R_LIFT, false>(f, a, false)), "lift");
+  a.E = f->BxB;
+  for (int l = 0; l < L; ++l) {
+    ColArgs c = column_args(f, l);
+    if (target) {
+      c.Hr = f->Hr[l];
+      c.Hi = f->Hi[l];
+    }
+    FNO_CUDA(run_column<false>(f, c, B, true), "spectral columns");
+    a.A = f->hb[l];
+    a.W = f->wbf + f->boff_Wt[l];
+    a.bias = f->theta + f->off_b[l];
+    a.zout = target ? f->z[l] : nullptr;
+    if (l + 1 < L) {
+      a.hb = f->hb[l + 1];
+      if (target) FNO_CUDA((run_row<R_FWD, true>(f, a, true)), "row layer");
+      else FNO_CUDA((run_row<R_FWD, false>(f, a, true)), "row layer");
+    } else {
+      a.Wq = f->theta + f->off_Wq;
+      a.bq = f->theta + f->off_bq;
+      a.out = out;
+      if (target) {
+        a.target = target;
+        a.dout = f->dout;
+        a.lpart = f->lpart;
+        a.hb = f->dzb;
+        a.C = f->BxTB;
+        FNO_CUDA((run_row<R_LAST_TRAIN, true>(f, a, true)), "last row layer");
+        loss_kernel<<<1, 256, 0, f->stream>>>(f->lpart, a.Q, 1.0 / (double)a.P, f->loss);
+        FNO_CUDA(cudaGetLastError(), "loss");
+      } else {
+        FNO_CUDA((run_row<R_LAST, false>(f, a, true)), "last row layer");
+      }
+    }
+  }
+  return TTSH_OK;
+}
+
+template <int AM, int DM>
+ttsh_status wgrad_partials(ttsh_fno* f, WgArgs a, int slot, int nout, int nw, float* gw, float* gb, WgReduceAll& red) {
+  a.chunk = (int)((a.P + f->nwblk - 1) / f->nwblk);
+  red.nblk = (int)((a.P + a.chunk - 1) / a.chunk);
+  a.part = f->wpart + (long long)slot * f->nwblk * (CW * CW + CW);
+  a.Wp = f->theta + f->off_Wp;
+  a.bp = f->theta + f->off_bp;
+  a.Wq = f->theta + f->off_Wq;
+  wgrad_kernel<AM, DM><<<red.nblk, 32 * kWgWarps, kWgSmem, f->stream>>>(a);
+  red.g[slot] = WgReduce{a.part, gw, gb, nout, nw};
+  FNO_CUDA(cudaGetLastError(), "weight gradient");
+  return TTSH_OK;
+}
+
+ttsh_status backward_fused(ttsh_fno* f, const float* x, int B) {
+  const int L = f->L, nmodes = 2 * f->m * f->m;
+  WgReduceAll red{};
+  WgArgs g{};
+  g.P = (long long)B * f->nn;
+  ttsh_status st;
+  constexpr int NO = CW * CW + CW;
+  // projection: dWq = z_{L-1}^T dout
+  g.A = f->z[L - 1];
+  g.D = f->dout;
+  if ((st = wgrad_partials<WA_RAW, WD_ONE>(f, g, L, CW + 1, CW, f->grad + f->off_Wq, f->grad + f->off_bq, red)) != TTSH_OK)
+    return st;
+  for (int l = L - 1; l >= 0; --l) {
+    // dW_l = h_l^T dz_l, with h_l = GELU(z_{l-1}) (the lift of x at l = 0) and, in the last
+    // layer, dz = dout Wq formed where they are read
+    const bool last = l + 1 == L;
+    float *gw = f->grad + f->off_W[l], *gb = f->grad + f->off_b[l];
+    g.A = l ? f->z[l - 1] : x;
+    g.D = last ? f->dout : f->dz;
+    if (l && last) st = wgrad_partials<WA_GELU, WD_OUTER>(f, g, l, NO, CW * CW, gw, gb, red);
+    else if (l) st = wgrad_partials<WA_GELU, WD_RAW>(f, g, l, NO, CW * CW, gw, gb, red);
+    else if (last) st = wgrad_partials<WA_LIFT, WD_OUTER>(f, g, l, NO, CW * CW, gw, gb, red);
+    else st = wgrad_partials<WA_LIFT, WD_RAW>(f, g, l, NO, CW * CW, gw, gb, red);
+    if (st != TTSH_OK) return st;
+    ColArgs c = column_args(f, l);
+    c.Hr = f->Yr;   // dY
+    c.Hi = f->Yi;
+    FNO_CUDA(run_column<true>(f, c, B, false), "spectral columns adjoint");
+    mode_wgrad_kernel<<<nmodes, 256, 0, f->stream>>>(f->Hr[l], f->Hi[l], f->Yr, f->Yi, nmodes, B, f->grad + f->off_Wr[l],
+                                                     f->grad + f->off_Wi[l]);
+    FNO_CUDA(cudaGetLastError(), "spectral weight gradient");
+    RowArgs a = row_args(f, B);
+    a.A = f->dzb;
+    a.W = f->wbf + f->boff_Wn[l];
+    a.E = f->FxTB;
+    a.dz = f->dz;
+    if (l > 0) {
+      a.C = f->BxTB;
+      a.zin = f->z[l - 1];
+      a.hb = f->dzb;
+      FNO_CUDA((run_row<R_BWD, true>(f, a, false)), "row layer adjoint");
+    } else {
+      FNO_CUDA((run_row<R_BWD_FIRST, true>(f, a, false)), "first row layer adjoint");
+    }
+  }
+  // lift: dWp = x^T dh_0
+  g.A = x;
+  g.D = f->dz;
+  if ((st = wgrad_partials<WA_X, WD_RAW>(f, g, L + 1, 5 * CW, 4 * CW, f->grad + f->off_Wp, f->grad + f->off_bp, red)) != TTSH_OK)
+    return st;
+  wgrad_reduce_all_kernel<<<dim3((NO + 7) / 8, L + 2), 256, 0, f->stream>>>(red);
+  FNO_CUDA(cudaGetLastError(), "weight gradient sums");
+  return TTSH_OK;
+}
+
 // Forward pass for B samples (x: B*n*n x cin); leaves activations for backward.
 ttsh_status forward_impl(ttsh_fno* f, const float* x, int B, float* out, const float* target, double* loss) {
+  if (f->fused) return forward_fused(f, x, B, out, target);
   cudaStream_t s = f->stream;
   const int n = f->n, C = f->C, m = f->m, L = f->L;
   const long long P = (long long)B * f->nn;
@@ -1134,6 +1412,7 @@ ttsh_status wgrad(ttsh_fno* f, const float* A, int ca, const float* D, int cd, l
 }
 
 ttsh_status backward_impl(ttsh_fno* f, const float* x, int B, const float* out) {
+  if (f->fused) return backward_fused(f, x, B);
   cudaStream_t s = f->stream;
   const int n = f->n, C = f->C, m = f->m, L = f->L;
   const long long P = (long long)B * f->nn;
@@ -1251,6 +1530,12 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
   const long long P = f->Pmax, PC = P * C;
   const long long sH = 2LL * m * m * C;   // floats per sample of kept modes
   f->nwblk = 512;
+  // the fused column kernels need their plan in shared memory
+  f->fused_columns = column_fwd_mix_smem(n) <= 220 * 1024 && row_dft_smem(n, m) <= 220 * 1024 && 2 * m <= 64 &&
+                     (2 * m) % JB == 0 && n % YB == 0;
+  f->tc_rows = n % 16 == 0 && n <= kXcMaxN && 2 * m <= 32;
+  f->fused = f->fused_columns && f->tc_rows;
+  f->cluster = n >= 32 ? 8 : 4;
   auto A = [&](auto** p, size_t bytes) {
     if (e == cudaSuccess) e = dalloc(f, p, bytes);
   };
@@ -1274,7 +1559,6 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
   f->hb.assign(L, nullptr);
   f->Hr.assign(L, nullptr);
   f->Hi.assign(L, nullptr);
-  for (int l = 0; l <= L; ++l) A(&f->h[l], PC * 4);
   for (int l = 0; l < L; ++l) {
     A(&f->z[l], PC * 4);
     A(&f->hb[l], PC * 2);
@@ -1285,21 +1569,27 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
   A(&f->Yr, f->Bmax * sH * 4);
   A(&f->Yi, f->Bmax * sH * 4);
   A(&f->Z, (long long)f->Bmax * n * 2 * m * C * 4);
-  A(&f->s, (PC > 2 * f->Bmax * sH ? PC : 2 * f->Bmax * sH) * 4);
-  A(&f->dh, PC * 4);
   A(&f->dz, PC * 4);
   A(&f->dzb, PC * 2);
-  A(&f->dspec, PC * 4);
   A(&f->dout, P * 4);
   A(&f->yo, P * 4);
-  A(&f->wpart, (long long)f->nwblk * (C * C + C) * 4);
-  A(&f->lpart, ((P + 255) / 256) * 8);
+  if (!f->fused) {
+    for (int l = 0; l <= L; ++l) A(&f->h[l], PC * 4);
+    A(&f->s, (PC > 2 * f->Bmax * sH ? PC : 2 * f->Bmax * sH) * 4);
+    A(&f->dh, PC * 4);
+    A(&f->dspec, PC * 4);
+  }
+  A(&f->wpart, (f->fused ? L + 2 : 1) * (long long)f->nwblk * (C * C + C) * 4);
+  const long long nlp = f->fused ? (long long)f->Bmax * n : (P + 255) / 256;   // partial sums of the loss
+  A(&f->lpart, nlp * 8);
   A(&f->tc_err, 64);
+  if (e == cudaSuccess) f->loss = reinterpret_cast<double*>(f->tc_err) + 1;
   if (e == cudaSuccess) e = cudaMemsetAsync(f->tc_err, 0, 64, f->stream);
   if (e != cudaSuccess) return cleanup(fno_cuda(e, "FNO allocation"));
-  // the fused column kernel needs its plan in shared memory
-  if (column_fwd_mix_smem(n) <= 220 * 1024 && row_dft_smem(n, m) <= 220 * 1024 && 2 * m <= 64 &&
-      (2 * m) % JB == 0 && n % YB == 0) {
+  if (f->fused) {
+    e = fused_setup(f);
+    if (e != cudaSuccess) return cleanup(fno_cuda(e, "layer kernel attribute"));
+  } else if (f->fused_columns) {
     e = cudaFuncSetAttribute(column_fwd_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              column_fwd_mix_smem(n));
     if (e == cudaSuccess)
@@ -1307,7 +1597,6 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(row_idft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, row_idft_smem(n, m));
     if (e != cudaSuccess) return cleanup(fno_cuda(e, "column kernel attribute"));
-    f->fused_columns = true;
   }
   // DFT matrices on the kept modes
   {
@@ -1353,10 +1642,9 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
       e = cudaMemcpy(bdst[i], bsrc[i]->data(), bsrc[i]->size() * 2, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cleanup(fno_cuda(e, "DFT matrices"));
-    if (n % 16 == 0 && n <= kXcMaxN && 2 * m <= 32) {
+    if (f->tc_rows && !f->fused) {
       e = cudaFuncSetAttribute(xcontract_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, xcontract_smem(n));
       if (e != cudaSuccess) return cleanup(fno_cuda(e, "row contraction attribute"));
-      f->tc_rows = true;
     }
   }
   // seeded initialisation: pointwise weights U(-1/sqrt(fan_in), 1/sqrt(fan_in)), biases 0,
@@ -1433,8 +1721,18 @@ ttsh_status ttsh_fno_loss_grad(ttsh_fno* f, const float* x, const float* target,
   if (grad_host) {
     FNO_CUDA(cudaMemcpyAsync(grad_host, f->grad, f->nparams * 4, cudaMemcpyDeviceToHost, f->stream), "get grad");
   }
-  FNO_CUDA(cudaStreamSynchronize(f->stream), "loss_grad");
-  if ((st = check_tc(f)) != TTSH_OK) return st;
+  if (f->fused) {   // the status word and the loss in one copy
+    double st2[2] = {0, 0};
+    FNO_CUDA(cudaMemcpyAsync(st2, f->tc_err, sizeof(st2), cudaMemcpyDeviceToHost, f->stream), "loss");
+    FNO_CUDA(cudaStreamSynchronize(f->stream), "loss_grad");
+    int h = 0;
+    memcpy(&h, st2, sizeof(h));
+    if (h) return check_tc(f);
+    l = st2[1];
+  } else {
+    FNO_CUDA(cudaStreamSynchronize(f->stream), "loss_grad");
+    if ((st = check_tc(f)) != TTSH_OK) return st;
+  }
   if (loss) *loss = l;
   return TTSH_OK;
 }
@@ -1443,10 +1741,11 @@ ttsh_status ttsh_fno_adam_step(ttsh_fno* f, float lr, float beta1, float beta2, 
   if (!f || !(lr > 0)) return fno_fail(TTSH_E_INVALID, "bad arguments");
   f->adam_t += 1;
   const float c1 = 1.f - powf(beta1, (float)f->adam_t), c2 = 1.f - powf(beta2, (float)f->adam_t);
-  adam_kernel<<<(unsigned)((f->nparams + 255) / 256), 256, 0, f->stream>>>(f->theta, f->grad, f->adam_m, f->adam_v,
-                                                                           f->nparams, lr, beta1, beta2, eps, c1, c2);
+  const long long msz2 = 4LL * f->m * f->m * f->C * f->C, lay = msz2 + CW * CW + CW, blay = msz2 + 2 * CW * CW;
+  adam_bf16_kernel<<<(unsigned)((f->nparams + 1023) / 1024), 256, 0, f->stream>>>(
+      (float4*)f->theta, (const float4*)f->grad, (float4*)f->adam_m, (float4*)f->adam_v, f->nparams, lr, beta1, beta2,
+      eps, c1, c2, f->off_Wr[0], lay, msz2, f->L, blay, f->wbf);
   FNO_CUDA(cudaGetLastError(), "adam");
-  FNO_CUDA(refresh_bf16(f), "adam");
   return TTSH_OK;
 }
 
