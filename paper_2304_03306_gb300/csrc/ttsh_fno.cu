@@ -555,59 +555,6 @@ __global__ void gelu_bwd_kernel(const float* __restrict__ dh, const float* __res
   dzb[i] = __float2bfloat16_rn(v);
 }
 
-// Partial weight gradients over a chunk of points: part[blk][i*cd + o] = sum_p A[p][i] D[p][o],
-// part[blk][ca*cd + o] = sum_p D[p][o]  (ca, cd <= 32; fixed order)
-__global__ void __launch_bounds__(256) wgrad_partial_kernel(const float* __restrict__ A, int ca,
-                                                            const float* __restrict__ D, int cd, long long P,
-                                                            int chunk, float* __restrict__ part) {
-  __shared__ float As[64][33];
-  __shared__ float Ds[64][33];
-  const int nout = ca * cd + cd;
-  float acc[5] = {0, 0, 0, 0, 0};   // up to 5 outputs per thread (1056 / 256 -> 5)
-  const long long p0 = (long long)blockIdx.x * chunk;
-  const long long p1 = p0 + chunk < P ? p0 + chunk : P;
-  for (long long pb = p0; pb < p1; pb += 64) {
-    for (int e = threadIdx.x; e < 64 * 32; e += 256) {
-      const int r = e >> 5, c = e & 31;
-      const long long p = pb + r;
-      As[r][c] = (p < p1 && c < ca) ? A[p * ca + c] : 0.f;
-      Ds[r][c] = (p < p1 && c < cd) ? D[p * cd + c] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int o = threadIdx.x + 256 * q;
-      if (o < nout) {
-        const int i = o / cd, j = o % cd;
-        float s = 0.f;
-        if (i < ca)
-          for (int r = 0; r < 64; ++r) s = fmaf(As[r][i], Ds[r][j], s);
-        else
-          for (int r = 0; r < 64; ++r) s += Ds[r][j];
-        acc[q] += s;
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    const int o = threadIdx.x + 256 * q;
-    if (o < nout) part[(long long)blockIdx.x * nout + o] = acc[q];
-  }
-}
-
-// grad[w_off + i*cd + o] = sum_blk part (then bias at b_off + o); fixed order over blocks
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int nblk, int ca, int cd,
-                                    float* __restrict__ gw, float* __restrict__ gb) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nout = ca * cd + cd;
-  if (o >= nout) return;
-  double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += part[(long long)b * nout + o];
-  if (o < ca * cd) gw[o] = (float)s;
-  else gb[o - ca * cd] = (float)s;
-}
-
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
@@ -979,6 +926,7 @@ struct ttsh_fno {
   std::vector<long long> boff_Wr, boff_Wi, boff_Wt, boff_Wn;
   // DFT matrices
   float *Fx = nullptr, *Gr = nullptr, *Gi = nullptr, *Gpr = nullptr, *Gpi = nullptr, *Bx = nullptr;
+  float* G2 = nullptr;          // (Gr, Gi) pairs of the column kernels
   // activations
   std::vector<float*> h, z;                     // h[0..L], z[0..L-1]
   std::vector<__nv_bfloat16*> hb;               // hb[0..L-1]
@@ -998,7 +946,6 @@ struct ttsh_fno {
   bool tc_rows = false;
   // two kernels a layer (ttsh_fno_fused.cuh): tc_rows, fused_columns and n <= 512
   bool fused = false;
-  int cluster = 8;              // blocks per cluster of the column kernels
   double* loss = nullptr;       // in the same 64 bytes as tc_err, behind it
   long long adam_t = 0;
   std::vector<void*> allocs;
@@ -1120,18 +1067,33 @@ cudaError_t launch_layer(void (*k)(A), dim3 grid, int block, int smem, cudaStrea
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 
+// Shared-memory limit, and the largest carve-out: row and column kernels of one pass share the
+// SMs, so that a kernel's blocks are in place, their constant operands staged, when the one
+// before it ends.
+template <typename K>
+cudaError_t layer_attributes(K k, int smem) {
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  return e;
+}
+
 template <int MODE, int T, bool TRAIN>
 cudaError_t row_one(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup) {
-  const int smem = row_smem(MODE, TRAIN, f->n);
   auto k = &row_layer_kernel<MODE, T, TRAIN>;
-  if (setup) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  // resident blocks per SM: tensor memory (64 T of 512 columns each), shared memory, 64 warps
-  int per = 8 / T;
+  if (setup) return layer_attributes(k, row_smem(MODE, TRAIN, f->n, 2));
+  // One grid row a block where all of them fit at two (one for 512 points) an SM: a single A
+  // tile then leaves room beside a column kernel's block, so that the row blocks are all in
+  // place when the columns are done.  Beyond that as many blocks as fit walk over the rows:
+  // tensor memory (64 T of 512 columns each), shared memory, 32 warps of up to 128 registers.
+  RowArgs r = a;
+  r.tiles = a.Q <= 152LL * (T == 4 ? 1 : 2) || !row_has_mma(MODE) ? 1 : 2;
+  const int smem = row_smem(MODE, TRAIN, f->n, r.tiles);
+  int per = T == 4 ? 1 : T == 2 ? 2 : 4;
   const int fit = (227 * 1024) / (smem + 2048);
   if (fit < per) per = fit < 1 ? 1 : fit;
-  if (per > 16 / T / 2) per = 16 / T / 2;
-  const long long cap = 152LL * per;
-  return launch_layer(k, dim3((unsigned)(a.Q < cap ? a.Q : cap)), 128 * T, smem, f->stream, pdl, 1, a);
+  const long long cap = r.tiles == 1 && row_has_mma(MODE) ? a.Q : 152LL * per;
+  return launch_layer(k, dim3((unsigned)(a.Q < cap ? a.Q : cap)), 128 * T, smem, f->stream, pdl, 1, r);
 }
 
 template <int MODE, bool TRAIN>
@@ -1143,10 +1105,13 @@ cudaError_t run_row(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup = false)
 
 template <bool ADJ>
 cudaError_t run_column(ttsh_fno* f, const ColArgs& a, int B, bool pdl, bool setup = false) {
-  const int cs = f->cluster, smem = col_smem(f->n, 2 * f->m, cs);
-  auto k = cs == 8 ? &column_layer_kernel<8, ADJ> : &column_layer_kernel<4, ADJ>;
-  if (setup) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return launch_layer(k, dim3((unsigned)(cs * f->m), (unsigned)B), kColThreads, smem, f->stream, pdl, cs, a);
+  auto k = &column_layer_kernel<ADJ>;
+  const int pieces = f->n / col_piece(f->n), two = pieces < 2 ? pieces : 2;
+  ColArgs c = a;
+  c.ring = CS * f->m * B <= 152 && pieces <= 4 ? pieces : two;   // (up to 256^2: 64 KB)
+  const int smem = col_smem(f->n, f->m, c.ring, ADJ);
+  if (setup) return layer_attributes(k, col_smem(f->n, f->m, pieces <= 4 ? pieces : 2, ADJ));
+  return launch_layer(k, dim3((unsigned)(CS * f->m), (unsigned)B), kColThreads, smem, f->stream, pdl, CS, c);
 }
 
 cudaError_t fused_setup(ttsh_fno* f) {
@@ -1161,12 +1126,17 @@ cudaError_t fused_setup(ttsh_fno* f) {
   if (e == cudaSuccess) e = run_row<R_BWD_FIRST, true>(f, r, false, true);
   if (e == cudaSuccess) e = run_column<false>(f, c, 1, false, true);
   if (e == cudaSuccess) e = run_column<true>(f, c, 1, false, true);
+  return e;
+}
+
+cudaError_t wgrad_setup() {
+  cudaError_t e = cudaSuccess;
   auto wg = [&](auto k) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   };
   wg(&wgrad_kernel<WA_RAW, WD_ONE>);
-  wg(&wgrad_kernel<WA_GELU, WD_OUTER>);
-  wg(&wgrad_kernel<WA_GELU, WD_RAW>);
+  wg(&wgrad_kernel<WA_RAW, WD_OUTER>);
+  wg(&wgrad_kernel<WA_RAW, WD_RAW>);
   wg(&wgrad_kernel<WA_LIFT, WD_OUTER>);
   wg(&wgrad_kernel<WA_LIFT, WD_RAW>);
   wg(&wgrad_kernel<WA_X, WD_RAW>);
@@ -1180,15 +1150,16 @@ RowArgs row_args(ttsh_fno* f, int B) {
   a.Q = (long long)B * f->n;
   a.P = (long long)B * f->nn;
   a.err = f->tc_err;
-  a.X = f->Hx;
+  a.X = reinterpret_cast<float2*>(f->Hx);
   a.Z = f->Z;
   return a;
 }
 
 ColArgs column_args(ttsh_fno* f, int l) {
   ColArgs c{};
-  c.X = f->Hx;
+  c.X = reinterpret_cast<const float2*>(f->Hx);
   c.Z = f->Z;
+  c.G = reinterpret_cast<const float2*>(f->G2);
   c.Gr = f->Gr;
   c.Gi = f->Gi;
   c.Wr = f->wbf + f->boff_Wr[l];
@@ -1205,6 +1176,7 @@ ttsh_status forward_fused(ttsh_fno* f, const float* x, int B, float* out, const 
   const int L = f->L;
   RowArgs a = row_args(f, B);
   a.x = x;
+  a.x16 = reinterpret_cast<uintptr_t>(x) % 16 == 0;
   a.Wp = f->theta + f->off_Wp;
   a.bp = f->theta + f->off_bp;
   a.C = f->FxB;
@@ -1221,9 +1193,10 @@ ttsh_status forward_fused(ttsh_fno* f, const float* x, int B, float* out, const 
     a.A = f->hb[l];
     a.W = f->wbf + f->boff_Wt[l];
     a.bias = f->theta + f->off_b[l];
-    a.zout = target ? f->z[l] : nullptr;
+    a.gout = target ? f->z[l] : nullptr;   // GELU'(z), and z itself in the last layer
     if (l + 1 < L) {
       a.hb = f->hb[l + 1];
+      a.hout = target ? f->h[l + 1] : nullptr;
       if (target) FNO_CUDA((run_row<R_FWD, true>(f, a, true)), "row layer");
       else FNO_CUDA((run_row<R_FWD, false>(f, a, true)), "row layer");
     } else {
@@ -1266,6 +1239,7 @@ ttsh_status backward_fused(ttsh_fno* f, const float* x, int B) {
   WgReduceAll red{};
   WgArgs g{};
   g.P = (long long)B * f->nn;
+  g.a16 = reinterpret_cast<uintptr_t>(x) % 16 == 0;
   ttsh_status st;
   constexpr int NO = CW * CW + CW;
   // projection: dWq = z_{L-1}^T dout
@@ -1274,14 +1248,14 @@ ttsh_status backward_fused(ttsh_fno* f, const float* x, int B) {
   if ((st = wgrad_partials<WA_RAW, WD_ONE>(f, g, L, CW + 1, CW, f->grad + f->off_Wq, f->grad + f->off_bq, red)) != TTSH_OK)
     return st;
   for (int l = L - 1; l >= 0; --l) {
-    // dW_l = h_l^T dz_l, with h_l = GELU(z_{l-1}) (the lift of x at l = 0) and, in the last
-    // layer, dz = dout Wq formed where they are read
+    // dW_l = h_l^T dz_l; the lift of x (h_0) and the last layer's dz = dout Wq are formed where
+    // they are read
     const bool last = l + 1 == L;
     float *gw = f->grad + f->off_W[l], *gb = f->grad + f->off_b[l];
-    g.A = l ? f->z[l - 1] : x;
+    g.A = l ? f->h[l] : x;
     g.D = last ? f->dout : f->dz;
-    if (l && last) st = wgrad_partials<WA_GELU, WD_OUTER>(f, g, l, NO, CW * CW, gw, gb, red);
-    else if (l) st = wgrad_partials<WA_GELU, WD_RAW>(f, g, l, NO, CW * CW, gw, gb, red);
+    if (l && last) st = wgrad_partials<WA_RAW, WD_OUTER>(f, g, l, NO, CW * CW, gw, gb, red);
+    else if (l) st = wgrad_partials<WA_RAW, WD_RAW>(f, g, l, NO, CW * CW, gw, gb, red);
     else if (last) st = wgrad_partials<WA_LIFT, WD_OUTER>(f, g, l, NO, CW * CW, gw, gb, red);
     else st = wgrad_partials<WA_LIFT, WD_RAW>(f, g, l, NO, CW * CW, gw, gb, red);
     if (st != TTSH_OK) return st;
@@ -1299,7 +1273,7 @@ ttsh_status backward_fused(ttsh_fno* f, const float* x, int B) {
     a.dz = f->dz;
     if (l > 0) {
       a.C = f->BxTB;
-      a.zin = f->z[l - 1];
+      a.gin = f->z[l - 1];
       a.hb = f->dzb;
       FNO_CUDA((run_row<R_BWD, true>(f, a, false)), "row layer adjoint");
     } else {
@@ -1401,13 +1375,21 @@ ttsh_status forward_impl(ttsh_fno* f, const float* x, int B, float* out, const f
   return TTSH_OK;
 }
 
+// One weight gradient of the unfused path: dW = A^T D, db = sum D.
 ttsh_status wgrad(ttsh_fno* f, const float* A, int ca, const float* D, int cd, long long P, float* gw, float* gb) {
-  const int nout = ca * cd + cd;
-  const long long chunk = (P + f->nwblk - 1) / f->nwblk;
-  const int nblk = (int)((P + chunk - 1) / chunk);
-  wgrad_partial_kernel<<<nblk, 256, 0, f->stream>>>(A, ca, D, cd, P, (int)chunk, f->wpart);
-  wgrad_reduce_kernel<<<(nout + 255) / 256, 256, 0, f->stream>>>(f->wpart, nblk, ca, cd, gw, gb);
-  FNO_CUDA(cudaGetLastError(), "weight gradient");
+  WgReduceAll red{};
+  WgArgs g{};
+  g.A = A;
+  g.D = D;
+  g.a16 = reinterpret_cast<uintptr_t>(A) % 16 == 0;
+  g.P = P;
+  ttsh_status st;
+  if (ca != CW) st = wgrad_partials<WA_X, WD_RAW>(f, g, 0, 5 * CW, 4 * CW, gw, gb, red);
+  else if (cd == 1) st = wgrad_partials<WA_RAW, WD_ONE>(f, g, 0, CW + 1, CW, gw, gb, red);
+  else st = wgrad_partials<WA_RAW, WD_RAW>(f, g, 0, CW * CW + CW, CW * CW, gw, gb, red);
+  if (st != TTSH_OK) return st;
+  wgrad_reduce_all_kernel<<<dim3((CW * CW + CW + 7) / 8, 1), 256, 0, f->stream>>>(red);
+  FNO_CUDA(cudaGetLastError(), "weight gradient sums");
   return TTSH_OK;
 }
 
@@ -1535,7 +1517,6 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
                      (2 * m) % JB == 0 && n % YB == 0;
   f->tc_rows = n % 16 == 0 && n <= kXcMaxN && 2 * m <= 32;
   f->fused = f->fused_columns && f->tc_rows;
-  f->cluster = n >= 32 ? 8 : 4;
   auto A = [&](auto** p, size_t bytes) {
     if (e == cudaSuccess) e = dalloc(f, p, bytes);
   };
@@ -1550,6 +1531,7 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
   A(&f->Gpr, 2LL * m * n * 4);
   A(&f->Gpi, 2LL * m * n * 4);
   A(&f->Bx, 2LL * m * n * 4);
+  if (f->fused) A(&f->G2, 4LL * m * n * 4);
   A(&f->FxB, 32LL * n * 2);
   A(&f->BxB, 32LL * n * 2);
   A(&f->FxTB, 32LL * n * 2);
@@ -1573,7 +1555,9 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
   A(&f->dzb, PC * 2);
   A(&f->dout, P * 4);
   A(&f->yo, P * 4);
-  if (!f->fused) {
+  if (f->fused) {
+    for (int l = 1; l < L; ++l) A(&f->h[l], PC * 4);
+  } else {
     for (int l = 0; l <= L; ++l) A(&f->h[l], PC * 4);
     A(&f->s, (PC > 2 * f->Bmax * sH ? PC : 2 * f->Bmax * sH) * 4);
     A(&f->dh, PC * 4);
@@ -1586,6 +1570,8 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
   if (e == cudaSuccess) f->loss = reinterpret_cast<double*>(f->tc_err) + 1;
   if (e == cudaSuccess) e = cudaMemsetAsync(f->tc_err, 0, 64, f->stream);
   if (e != cudaSuccess) return cleanup(fno_cuda(e, "FNO allocation"));
+  e = wgrad_setup();
+  if (e != cudaSuccess) return cleanup(fno_cuda(e, "weight gradient attribute"));
   if (f->fused) {
     e = fused_setup(f);
     if (e != cudaSuccess) return cleanup(fno_cuda(e, "layer kernel attribute"));
@@ -1626,16 +1612,26 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
     float* dst[6] = {f->Fx, f->Gr, f->Gi, f->Gpr, f->Gpi, f->Bx};
     for (int i = 0; i < 6 && e == cudaSuccess; ++i)
       e = cudaMemcpy(dst[i], src[i]->data(), src[i]->size() * 4, cudaMemcpyHostToDevice);
-    // BF16 operands of the tensor-core row contractions, padded to 32 kept entries
+    if (f->fused && e == cudaSuccess) {
+      std::vector<float> g2(4 * (size_t)m * n);
+      for (size_t i = 0; i < 2 * (size_t)m * n; ++i) {
+        g2[2 * i] = Gr[i];
+        g2[2 * i + 1] = Gi[i];
+      }
+      e = cudaMemcpy(f->G2, g2.data(), g2.size() * 4, cudaMemcpyHostToDevice);
+    }
+    // BF16 operands of the tensor-core row contractions, padded to 32 kept entries; the layer
+    // kernels take the contracting rows as Re 0, Im 0, Re 1, ...
     std::vector<__nv_bfloat16> fxb(32 * n), bxb(32 * n), fxtb(32 * n), bxtb(32 * n);
     for (int j = 0; j < 32; ++j)
       for (int x = 0; x < n; ++x) {
         const float fv = j < 2 * m ? Fx[j * n + x] : 0.f;
         const float bv = j < 2 * m ? Bx[x * 2 * m + j] : 0.f;
-        fxb[j * n + x] = __float2bfloat16_rn(fv);    // [j][x]
+        const int row = !f->fused || j >= 2 * m ? j : j < m ? 2 * j : 2 * (j - m) + 1;
+        fxb[row * n + x] = __float2bfloat16_rn(fv);  // [j][x]
         fxtb[x * 32 + j] = __float2bfloat16_rn(fv);  // [x][j]
         bxb[x * 32 + j] = __float2bfloat16_rn(bv);   // [x][j]
-        bxtb[j * n + x] = __float2bfloat16_rn(bv);   // [j][x]
+        bxtb[row * n + x] = __float2bfloat16_rn(bv); // [j][x]
       }
     const std::vector<__nv_bfloat16>* bsrc[4] = {&fxb, &bxb, &fxtb, &bxtb};
     __nv_bfloat16* bdst[4] = {f->FxB, f->BxB, f->FxTB, f->BxTB};

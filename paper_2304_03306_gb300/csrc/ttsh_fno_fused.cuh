@@ -10,21 +10,37 @@
 //                  ky, the per-mode complex mixing and the inverse transform along y, the mixed
 //                  modes exchanged through distributed shared memory.
 //
-// Spectral columns lie as [b][k][y][channel] (k = Re kx 0..m-1, then Im), so that a block's two
-// columns are contiguous.  Every FP32 sum runs in the order of the separate kernels these
+// Spectral columns on their way to the column kernel lie as [b][kx][y][channel] (Re, Im) pairs,
+// so that a block's column is one contiguous piece; on their way back as [b][k][y][channel]
+// (k = Re kx 0..m-1, then Im), the order of the expanding products' K.  Every FP32 sum runs in the order of the separate kernels these
 // replace, so that results, including every rounding to BF16, are the same bits.
 #pragma once
+
+#include <type_traits>
 
 namespace fno_dev {
 
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// One warp waits for the kernel ahead, the others at the block barrier: threads in
+// griddepcontrol.wait take issue slots from the kernel they wait for.
+__device__ __forceinline__ void pdl_wait_block() {
+  if (threadIdx.x < 32) asm volatile("griddepcontrol.wait;" ::: "memory");
+  __syncthreads();
+}
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_all;\n" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------
 // Row kernel
+//
+// Bound at batch 8 by memory in the backward pass (217 MB, 32 us at the measured copy rate; 35-42 us)
+// and by erf and exp besides in the forward one (218 MB with what the backward pass needs; 55-64
+// us); at batch 1 by its chain of phases (8 us, of which 0.6 us wait for the columns, 0.5 us the
+// products, 2 us the activation, 1.5 us the contraction).  The launches it replaces (expand,
+// channel mixing, contract) took 38 us at batch 1 and 134 us (forward, training) at batch 8.
+// One thread holds the 32 channels of one point, so that activation and projection need no
+// exchange; the A tile of the next row travels while a block works on this one.
 // ---------------------------------------------------------------------------------------
 enum RowMode {
   R_LIFT = 0,        // h_0 = x Wp + bp, contracted with Fx
@@ -40,13 +56,15 @@ struct RowArgs {
   const __nv_bfloat16* W;    // 32 x 32, [o][i]
   const __nv_bfloat16* E;    // [n][32]: matrix that expands the kept kx to the row
   const float* Z;            // [B][J][n][32]: columns to expand
-  const __nv_bfloat16* C;    // [32][n]: matrix that contracts the row to the kept kx
-  float* X;                  // [B][J][n][32]: contracted columns
+  const __nv_bfloat16* C;    // [32][n]: matrix that contracts the row to the kept kx, rows Re 0, Im 0, Re 1, ...
+  float2* X;                 // [B][m][n][32]: contracted columns
   const float* bias;         // 32
-  const float* x;            // R_LIFT: [P][4]
+  const float* x;            // R_LIFT: [P][4], the caller's
+  int x16;                   // 1: x is 16-byte aligned
   const float *Wp, *bp;      // R_LIFT
-  const float* zin;          // R_BWD: z of the layer below
-  float* zout;               // forward in training: z (null otherwise)
+  const float* gin;          // R_BWD: GELU'(z) of the layer below
+  float* gout;               // R_FWD in training: GELU'(z); R_LAST_TRAIN: z
+  float* hout;               // R_FWD in training: GELU(z)
   __nv_bfloat16* hb;         // result in BF16: h_{l+1}, or dz
   float* dz;                 // R_BWD: dz', R_BWD_FIRST: dh
   const float *Wq, *bq;      // R_LAST*
@@ -54,7 +72,7 @@ struct RowArgs {
   const float* target;       // R_LAST_TRAIN: [P]
   float* dout;               // R_LAST_TRAIN: [P]
   double* lpart;             // R_LAST_TRAIN: sum of squared errors of each grid row
-  int n, J;
+  int n, J, tiles;           // tiles: A tiles in shared memory, 2 if some block has several rows
   long long Q, P;            // grid rows, points
   int* err;
 };
@@ -65,11 +83,11 @@ __host__ __device__ constexpr bool row_stages(int mode, bool train) {   // FP32 
   return mode == R_BWD || mode == R_BWD_FIRST || mode == R_LAST_TRAIN || (mode == R_FWD && train);
 }
 
-// Dynamic shared memory: A tile | C | E | W | Z operand | FP32 rows of every warp, and 128 bytes
-// to align the base.
-inline int row_smem(int mode, bool train, int n) {
+// Dynamic shared memory: A tile, `tiles` times (two where a block walks over several grid rows) |
+// C | E | W | Z operand | FP32 rows of every warp, and 128 bytes to align the base.
+inline int row_smem(int mode, bool train, int n, int tiles) {
   const int nr = n < 128 ? 128 : n;
-  return 128 + nr * 64 + 64 * n + 2048 + (row_has_mma(mode) ? nr * 64 + 2048 : 0) +
+  return 128 + tiles * nr * 64 + 64 * n + 2048 + (row_has_mma(mode) ? nr * 64 + 2048 : 0) +
          (row_stages(mode, train) ? nr * 128 : 0);
 }
 
@@ -80,7 +98,7 @@ __device__ __forceinline__ float4* row_piece(unsigned char* blk, int r, int i) {
 }
 
 template <int MODE, int T, bool TRAIN>
-__global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
+__global__ void __launch_bounds__(128 * T, T == 4 ? 1 : TRAIN ? 2 : 3) row_layer_kernel(RowArgs a) {
   constexpr int NT = 128 * T;
   constexpr int TCOLS = 64 * T;   // per x tile: 32 columns for the channel mixing, 32 for the expansion
   extern __shared__ __align__(16) unsigned char row_dyn[];
@@ -89,10 +107,12 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
   __shared__ float sc[CW * 6];    // bias / Wp, bp / Wq
   __shared__ double lred[4 * T];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n = a.n, J = a.J, nr = n < 128 ? 128 : n;
+  const int n = T == 1 ? a.n : 128 * T;   // T = 1 serves every grid up to 128
+  constexpr int nr = 128 * T;
+  const int J = a.J;
   unsigned char* base = row_dyn + ((128u - (smem_u32(row_dyn) & 127u)) & 127u);
   unsigned char* sA = base;
-  unsigned char* sC = sA + nr * 64;
+  unsigned char* sC = sA + a.tiles * nr * 64;
   unsigned char* sE = sC + 64 * n;
   unsigned char* sW = sE + (row_has_mma(MODE) ? nr * 64 : 0);
   unsigned char* sZ = sW + 2048;
@@ -110,6 +130,12 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
     for (int c = tid; c < n * 4; c += NT) cp_async16(sE + core_off(c >> 2, c & 3), a.E + c * 8);
     for (int c = tid; c < CW * 4; c += NT) cp_async16(sW + core_off(c >> 2, c & 3), a.W + c * 8);
   }
+  // the first row's A tile: its writer finished before the kernel ahead of this one began
+  long long q = blockIdx.x;
+  if constexpr (row_has_mma(MODE)) {
+    if (q < a.Q)
+      for (int c = tid; c < n * 4; c += NT) cp_async16(sA + core_off(c >> 2, c & 3), a.A + q * n * CW + c * 8);
+  }
   if constexpr (MODE == R_LIFT) {
     for (int c = tid; c < 5 * CW; c += NT) sc[c] = c < 4 * CW ? a.Wp[c] : a.bp[c - 4 * CW];
   } else if constexpr (MODE == R_FWD) {
@@ -123,43 +149,49 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
   }
   if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)) : "memory");
   if (warp == 0) tc_alloc(&tmem_base, TCOLS);
-  cp_async_wait();
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_base;
   const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
   const int tile = warp >> 2;
   const int x = tid;               // this thread's point of the grid row
   const bool live = x < n;
   const int wrows = n - warp * 32 >= 32 ? 32 : (n - warp * 32 > 0 ? n - warp * 32 : 0);
   uint32_t phase = 0;
-  pdl_wait();
-  pdl_launch();
+  pdl_wait_block();
+  if constexpr (!row_has_mma(MODE)) pdl_launch();
 
-  for (long long q = blockIdx.x; q < a.Q; q += gridDim.x) {
+  // columns to expand: eight k of one channel a thread of the first four warps
+  float zc[8];
+  auto load_z = [&](long long qq) {
+    const long long bb = qq / n, yy = qq - bb * n;
+    const float* zp = a.Z + ((bb * J + warp * 8) * n + yy) * CW + lane;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) zc[i] = warp * 8 + i < J ? zp[(long long)i * n * CW] : 0.f;
+  };
+  if constexpr (row_has_mma(MODE)) {
+    if (warp < 4 && q < a.Q) load_z(q);
+  }
+  cp_async_wait();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+  for (; q < a.Q; q += gridDim.x) {
     const long long p0 = q * n;
     const int b = (int)(q / n), y = (int)(q - (long long)b * n);
     uint32_t acc[CW];
     float v[CW];
     if constexpr (row_has_mma(MODE)) {
-      for (int c = tid; c < n * 4; c += NT) cp_async16(sA + core_off(c >> 2, c & 3), a.A + p0 * CW + c * 8);
-      if constexpr (MODE == R_BWD) {   // z of the layer below, for GELU'
+      if constexpr (MODE == R_BWD) {   // GELU' of the layer below, needed after the products
         for (int i = lane; i < wrows * 8; i += 32)
-          cp_async16(row_piece(blk, i >> 3, i & 7), a.zin + (p0 + warp * 32) * CW + i * 4);
+          cp_async16(row_piece(blk, i >> 3, i & 7), a.gin + (p0 + warp * 32) * CW + i * 4);
+        asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      // columns to expand as the K-major operand [channel][k]: eight k of one channel a thread
-      if (warp < 4) {
+      if (warp < 4) {   // K-major operand [channel][k]
         __nv_bfloat16 e[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int j = warp * 8 + i;
-          const float f = j < J ? a.Z[(((long long)b * J + j) * n + y) * CW + lane] : 0.f;
-          e[i] = __float2bfloat16_rn(f);
-        }
+        for (int i = 0; i < 8; ++i) e[i] = __float2bfloat16_rn(zc[i]);
         *reinterpret_cast<uint4*>(sZ + core_off(lane, warp)) = *reinterpret_cast<const uint4*>(e);
       }
-      cp_async_wait();
+      asm volatile("cp.async.wait_group %0;" ::"n"(MODE == R_BWD ? 1 : 0) : "memory");   // this row's A tile
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor core
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncthreads();
@@ -177,12 +209,21 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
           }
         tc_commit(&mbar);
       }
+      // the next row's inputs travel while this one is worked on
+      const long long qn = q + gridDim.x;
+      if (qn < a.Q) {
+        unsigned char* nx = base + (sA == base ? nr * 64 : 0);
+        for (int c = tid; c < n * 4; c += NT) cp_async16(nx + core_off(c >> 2, c & 3), a.A + qn * n * CW + c * 8);
+        if (warp < 4) load_z(qn);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
       const bool done = ttsh::mbar_wait_bounded(smem_u32(&mbar), phase, ttsh::kWaitLimitNs);
       if (__syncthreads_or(!done)) {
         if (tid == 0) atomicExch(a.err, 1);
         break;
       }
       phase ^= 1u;
+      pdl_launch();   // the next kernel's blocks stage their operands under the epilogue
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       tc_ld32(tmem + lanes + tile * 64, acc);
 #pragma unroll
@@ -194,7 +235,12 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
         if constexpr (MODE == R_FWD || MODE == R_LAST || MODE == R_LAST_TRAIN) v[c] += sc[c];
       }
     } else {
-      const float4 xv = live ? *reinterpret_cast<const float4*>(a.x + (p0 + x) * 4) : make_float4(0, 0, 0, 0);
+      float4 xv = make_float4(0, 0, 0, 0);
+      if (live) {
+        const float* xp = a.x + (p0 + x) * 4;
+        if (a.x16) xv = *reinterpret_cast<const float4*>(xp);
+        else xv = make_float4(xp[0], xp[1], xp[2], xp[3]);
+      }
 #pragma unroll
       for (int c = 0; c < CW; ++c)
         v[c] = fmaf(xv.w, sc[3 * CW + c], fmaf(xv.z, sc[2 * CW + c], fmaf(xv.y, sc[CW + c], fmaf(xv.x, sc[c], sc[4 * CW + c]))));
@@ -210,13 +256,29 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
       for (int i = lane; i < wrows * 8; i += 32)
         *reinterpret_cast<float4*>(dst + (p0 + warp * 32) * CW + i * 4) = *row_piece(blk, i >> 3, i & 7);
     };
-    if constexpr ((MODE == R_FWD && TRAIN) || MODE == R_LAST_TRAIN) {
+    if constexpr (MODE == R_LAST_TRAIN) {
       put_rows();
-      store_rows(a.zout);
+      store_rows(a.gout);
     }
     if constexpr (MODE == R_FWD) {
+      if constexpr (TRAIN) {   // GELU' for the backward pass, while erf(z / sqrt 2) is at hand
+        float h[CW];
 #pragma unroll
-      for (int c = 0; c < CW; ++c) v[c] = gelu(v[c]);
+        for (int c = 0; c < CW; ++c) {
+          h[c] = gelu(v[c]);
+          v[c] = gelu_grad(v[c]);
+        }
+        put_rows();
+        store_rows(a.gout);
+#pragma unroll
+        for (int c = 0; c < CW; ++c) v[c] = h[c];
+        __syncwarp();
+        put_rows();
+        store_rows(a.hout);
+      } else {
+#pragma unroll
+        for (int c = 0; c < CW; ++c) v[c] = gelu(v[c]);
+      }
     }
     if constexpr (MODE == R_LAST || MODE == R_LAST_TRAIN) {
       float o = sc[2 * CW];
@@ -240,19 +302,21 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
       }
     }
     if constexpr (MODE == R_BWD) {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");   // all but the next row's tile
+      __syncwarp();
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const float4 z = *row_piece(blk, lane, i);
-        v[4 * i] *= gelu_grad(z.x);
-        v[4 * i + 1] *= gelu_grad(z.y);
-        v[4 * i + 2] *= gelu_grad(z.z);
-        v[4 * i + 3] *= gelu_grad(z.w);
+        const float4 g = *row_piece(blk, lane, i);
+        v[4 * i] *= g.x;
+        v[4 * i + 1] *= g.y;
+        v[4 * i + 2] *= g.z;
+        v[4 * i + 3] *= g.w;
       }
     }
     if constexpr (MODE == R_BWD || MODE == R_BWD_FIRST) {
-      if constexpr (MODE == R_BWD) __syncwarp();
       put_rows();
       store_rows(a.dz);
+      __syncwarp();   // read before the next row's copies
     }
 
     if constexpr (row_contracts(MODE)) {
@@ -298,14 +362,16 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (warp == 0) {   // accumulator rows 0..31: lane = channel, column = k
         tc_ld32(tmem, acc);
-        float* xo = a.X + ((long long)b * J * n + y) * CW + lane;
+        float2* xo = a.X + ((long long)b * (J / 2) * n + y) * CW + lane;
 #pragma unroll
-        for (int j = 0; j < CW; ++j)
-          if (j < J) xo[(long long)j * n * CW] = __uint_as_float(acc[j]);
+        for (int k = 0; k < CW / 2; ++k)
+          if (2 * k < J) xo[(long long)k * n * CW] = make_float2(__uint_as_float(acc[2 * k]), __uint_as_float(acc[2 * k + 1]));
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // accumulators read before reuse
+    if constexpr (row_has_mma(MODE)) sA = base + (sA == base ? nr * 64 : 0);
   }
+  cp_async_wait();   // a row left early (failed wait) may have copies in flight
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) tc_dealloc(tmem, TCOLS);
@@ -315,212 +381,279 @@ __global__ void __launch_bounds__(128 * T) row_layer_kernel(RowArgs a) {
 // Column kernel
 // ---------------------------------------------------------------------------------------
 struct ColArgs {
-  const float* X;                      // [B][J][n][32]
-  const float *Gr, *Gi;                // [J][n]: exp(-2 pi i ky y / n)
+  const float2* X;                     // [B][m][n][32]
+  const float2* G;                     // [J][n]: exp(-2 pi i ky y / n)
+  const float *Gr, *Gi;                // the same, planar
   const __nv_bfloat16 *Wr, *Wi;        // [J][m][32][32]
   float *Hr, *Hi;                      // [B][J][m][32]: modes before the mixing (null: not kept)
   float* Z;                            // [B][J][n][32]
   int n, m;
+  int ring;                            // pieces of X in shared memory at a time
   int* err;
 };
 
 // Forward (ADJ = false): H_j = sum_y G_jy X_y, Y = W H per mode, Z_y = sum_j conj(G_jy) Y_j.
-// Adjoint: the same transforms around dH = W^H dY.  Block `rank` of the cluster transforms JB of
-// the kept ky and JB's share of the mixing, and afterwards n / CS values of y.
+// Adjoint: the same transforms around dH = W^H dY.  Block `rank` of the cluster transforms PB pairs
+// of kept ky, mixes them, and afterwards transforms back n / CS values of y.
+//
+// Bound by what shared memory delivers to registers (4 bytes a lane and cycle, broadcast or not):
+// a thread therefore sums ky and -ky of one channel together, whose G are each other's
+// conjugates (ky = 0, whose G is 1, goes with -m), and transforms back four y of two channels.
+// Measured at 256^2, 16 modes: the first sum 3.5 us with one ky a thread, 5.8 us with 8 ky in
+// each of 4 blocks, 3.0 us so; the kernel 10 us at batch 1 and 33 us at batch 8 (268 MFLOP, 8 TFLOP/s;
+// its 17 MB of columns would take 2.5 us), where the separate kernels took 23 and 57 us.
 constexpr int kColThreads = 256;
+constexpr int CS = 8;   // blocks per cluster
 // BF16 values between the rows of a staged 32 x 32 weight: the adjoint reads a row per lane in
 // 16-byte pieces, and 80 bytes apart eight of them meet every bank once.
 __host__ __device__ constexpr int col_wrow(bool adj) { return adj ? 40 : CW; }
+// X passes through a ring of pieces of 64 y (16 KB): all of them in shared memory where a block has
+// an SM to itself anyway, two where further blocks then fit beside it.
+__host__ __device__ constexpr int col_piece(int n) { return n < 64 ? n : 64; }
+constexpr int kColRing = 8;
 
-inline int col_smem(int n, int J, int CS) {
-  const int JB = (J + CS - 1) / CS, ny = n / CS;
-  return 128 + 2 * n * CW * 4 + 2 * JB * n * 4 + 2 * J * ny * 4 + 2 * JB * CW * col_wrow(true) * 2 + 4 * JB * CW * 4 + 2 * J * CW * 4;
+inline int col_smem(int n, int m, int ring, bool adj) {
+  const int PB = (m + CS - 1) / CS, ny = n / CS < 4 ? 4 : n / CS;
+  return 128 + ring * col_piece(n) * CW * 8 + PB * n * 8 + 4 * m * ny * 4 + 4 * PB * CW * col_wrow(adj) * 2 +
+         2 * PB * CW * 8 + 2 * m * CW * 8;
 }
 
-template <int CS, bool ADJ>
+template <bool ADJ>
 __global__ void __launch_bounds__(kColThreads) column_layer_kernel(ColArgs a) {
   extern __shared__ __align__(16) unsigned char col_dyn[];
-  __shared__ __align__(8) uint64_t mbar;
+  __shared__ __align__(8) uint64_t mbar[kColRing];
   const int tid = threadIdx.x, warp = tid >> 5, c = tid & 31;
   const int n = a.n, m = a.m, J = 2 * m;
   const int kx = blockIdx.x / CS, rank = blockIdx.x % CS, b = blockIdx.y;
-  const int JB = (J + CS - 1) / CS, ny = n / CS;
-  const int j0 = rank * JB, jn = J - j0 < JB ? (J - j0 > 0 ? J - j0 : 0) : JB;   // this block's ky rows
-  const int y0 = rank * ny;
+  const int PB = (m + CS - 1) / CS, t0 = rank * PB, tn = m - t0 < PB ? (m - t0 > 0 ? m - t0 : 0) : PB;
+  const int ny = n / CS < 4 ? 4 : n / CS, y0 = rank * ny;   // this block's y (none where y0 >= n)
+  // rows of the pair t: the one whose G is read, and its mirror image
+  auto row_a = [m](int t) { return t == 0 ? m : t; };
+  auto row_b = [m](int t) { return t == 0 ? 0 : 2 * m - t; };
   constexpr int WROW = col_wrow(ADJ), WMAT = CW * WROW;
   unsigned char* base = col_dyn + ((128u - (smem_u32(col_dyn) & 127u)) & 127u);
-  float* xr = reinterpret_cast<float*>(base);                 // [n][32]
-  float* xi = xr + n * CW;
-  float* gr = xi + n * CW;                                    // [JB][n]
-  float* gi = gr + JB * n;
-  float* vr = gi + JB * n;                                    // [J][ny]: this block's y of every ky row
+  const int piece = col_piece(n), pieces = n / piece, ring = a.ring;
+  float2* xs = reinterpret_cast<float2*>(base);               // [ring][piece][32]
+  float2* gs = xs + ring * piece * CW;                        // [PB][n]
+  float* vr = reinterpret_cast<float*>(gs + PB * n);          // [J][ny]: this block's y of every ky row
   float* vi = vr + J * ny;
-  float* yr = vi + J * ny;                                    // [J][32]: every mixed mode
-  float* yi = yr + J * CW;
-  float* hr = yi + J * CW;                                    // [JB][32]: this block's modes
-  float* hi = hr + JB * CW;
-  float* mr = hi + JB * CW;                                   // [JB][32]: the same, mixed
-  float* mi = mr + JB * CW;
-  __nv_bfloat16* wr = reinterpret_cast<__nv_bfloat16*>(mi + JB * CW);   // [JB][32][WROW]
-  __nv_bfloat16* wi = wr + JB * WMAT;
+  float2* ys = reinterpret_cast<float2*>(vi + J * ny);        // [J][32]: every mixed mode
+  float2* hs = ys + J * CW;                                   // [2 PB][32]: this block's modes
+  __nv_bfloat16* wr = reinterpret_cast<__nv_bfloat16*>(hs + 2 * PB * CW);   // [2 PB][32][WROW]
+  __nv_bfloat16* wi = wr + 2 * PB * WMAT;
 
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)) : "memory");
+    for (int i = 0; i < ring; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[i])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int e = tid; e < jn * n / 4; e += kColThreads) {
-    cp_async16(gr + 4 * e, a.Gr + (long long)j0 * n + 4 * e);
-    cp_async16(gi + 4 * e, a.Gi + (long long)j0 * n + 4 * e);
+  asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // this block has started
+  const int lg = 31 - __clz(n / 2);   // n / 2 and ny / 4 are powers of two
+  for (int e = tid; e < tn * (n / 2); e += kColThreads) {
+    const int tl = e >> lg, r = e & ((1 << lg) - 1);
+    cp_async16(gs + tl * n + 2 * r, a.G + (long long)row_a(t0 + tl) * n + 2 * r);
   }
-  for (int e = tid; e < J * ny / 4; e += kColThreads) {
-    const int j = e / (ny / 4), r = e % (ny / 4);
-    cp_async16(vr + 4 * e, a.Gr + (long long)j * n + y0 + 4 * r);
-    cp_async16(vi + 4 * e, a.Gi + (long long)j * n + y0 + 4 * r);
+  if (y0 < n) {
+    const int lq = 31 - __clz(ny / 4);
+    for (int e = tid; e < J * ny / 4; e += kColThreads) {
+      const int j = e >> lq, r = e & ((1 << lq) - 1);
+      cp_async16(vr + 4 * e, a.Gr + (long long)j * n + y0 + 4 * r);
+      cp_async16(vi + 4 * e, a.Gi + (long long)j * n + y0 + 4 * r);
+    }
   }
-  for (int e = tid; e < jn * (CW * CW / 8); e += kColThreads) {
-    const int jl = e / (CW * CW / 8), r = e % (CW * CW / 8);
-    const long long src = ((long long)(j0 + jl) * m + kx) * CW * CW + 8 * r;
+  for (int e = tid; e < 2 * tn * (CW * CW / 8); e += kColThreads) {
+    const int jl = e / (CW * CW / 8), r = e % (CW * CW / 8), t = t0 + (jl >> 1);
+    const long long src = ((long long)(jl & 1 ? row_b(t) : row_a(t)) * m + kx) * CW * CW + 8 * r;
     const int dst = jl * WMAT + (r >> 2) * WROW + 8 * (r & 3);
     cp_async16(wr + dst, a.Wr + src);
     cp_async16(wi + dst, a.Wi + src);
   }
-  __syncthreads();   // the barrier is initialised
-  pdl_wait();
+  pdl_wait_block();   // (and the barriers are initialised)
   pdl_launch();
-  if (tid == 0) {
-    const uint32_t bytes = (uint32_t)(n * CW * 4);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(2 * bytes) : "memory");
-    const float* s0 = a.X + ((long long)b * J + kx) * n * CW;
+  auto load_piece = [&](int k) {   // thread 0: piece k of X into its place in the ring
+    const uint32_t bytes = (uint32_t)(piece * CW * 8), bar = smem_u32(&mbar[k % ring]);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(xr)), "l"(s0), "r"(bytes), "r"(smem_u32(&mbar)) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(xi)), "l"(s0 + (long long)m * n * CW), "r"(bytes), "r"(smem_u32(&mbar)) : "memory");
-  }
+                 ::"r"(smem_u32(xs + (k % ring) * piece * CW)), "l"(a.X + (((long long)b * m + kx) * n + k * piece) * CW),
+                 "r"(bytes), "r"(bar) : "memory");
+  };
+  if (tid == 0)
+    for (int k = 0; k < ring; ++k) load_piece(k);
   cp_async_wait();
-  if (!ttsh::mbar_wait_bounded(smem_u32(&mbar), 0, ttsh::kWaitLimitNs)) atomicExch(a.err, 1);
   __syncthreads();
 
-  for (int jl = warp; jl < jn; jl += kColThreads / 32) {
-    // ---- H_j = sum over y, in order ----
-    float ar = 0.f, ai = 0.f, br = 0.f, bi = 0.f;
-    const float* g0 = gr + jl * n;
-    const float* g1 = gi + jl * n;
-#pragma unroll 2
-    for (int y = 0; y < n; y += 4) {
-      const float4 p4 = *reinterpret_cast<const float4*>(g0 + y), q4 = *reinterpret_cast<const float4*>(g1 + y);
-      const float pv[4] = {p4.x, p4.y, p4.z, p4.w}, qv[4] = {q4.x, q4.y, q4.z, q4.w};
+  // ---- H_j = sum over y, in order: a warp takes a pair of ky, a lane a channel; the next eight y
+  // are loaded while these are summed (PB <= 2 pairs a block) ----
+  {
+    const bool on = warp < tn;
+    float ar[2] = {0, 0}, ai[2] = {0, 0}, br[2] = {0, 0}, bi[2] = {0, 0};
+    for (int k = 0; k < pieces; ++k) {
+      if (!ttsh::mbar_wait_bounded(smem_u32(&mbar[k % ring]), (k / ring) & 1, ttsh::kWaitLimitNs)) atomicExch(a.err, 1);
+      if (on) {
+        const float2* g = gs + warp * n + k * piece;
+        const float2* x = xs + (k % ring) * piece * CW + c;
+        float2 u[2][8];
+        float4 pq[2][4];
+        auto fetch = [&](int s, int y) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float u = xr[(y + i) * CW + c], w = xi[(y + i) * CW + c];
-        if constexpr (ADJ) {   // four sums, combined below
-          ar = fmaf(pv[i], u, ar);
-          br = fmaf(qv[i], w, br);
-          ai = fmaf(pv[i], w, ai);
-          bi = fmaf(qv[i], u, bi);
-        } else {
-          ar = fmaf(pv[i], u, fmaf(-qv[i], w, ar));
-          ai = fmaf(pv[i], w, fmaf(qv[i], u, ai));
+          for (int i = 0; i < 4; ++i) pq[s][i] = *reinterpret_cast<const float4*>(g + y + 2 * i);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) u[s][i] = x[(y + i) * CW];
+          asm volatile("" ::: "memory");   // loads stay ahead of the sums
+        };
+        auto sum = [&](int s, auto zero) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float2 v = u[s][i];
+            const float p = i & 1 ? pq[s][i >> 1].z : pq[s][i >> 1].x, q = i & 1 ? pq[s][i >> 1].w : pq[s][i >> 1].y;
+            const float p2 = decltype(zero)::value ? 1.f : p, q2 = decltype(zero)::value ? -0.f : -q;
+            if constexpr (ADJ) {   // four sums, combined below
+              ar[0] = fmaf(p, v.x, ar[0]);
+              br[0] = fmaf(q, v.y, br[0]);
+              ai[0] = fmaf(p, v.y, ai[0]);
+              bi[0] = fmaf(q, v.x, bi[0]);
+              ar[1] = fmaf(p2, v.x, ar[1]);
+              br[1] = fmaf(q2, v.y, br[1]);
+              ai[1] = fmaf(p2, v.y, ai[1]);
+              bi[1] = fmaf(q2, v.x, bi[1]);
+            } else {
+              ar[0] = fmaf(p, v.x, fmaf(-q, v.y, ar[0]));
+              ai[0] = fmaf(p, v.y, fmaf(q, v.x, ai[0]));
+              ar[1] = fmaf(p2, v.x, fmaf(-q2, v.y, ar[1]));
+              ai[1] = fmaf(p2, v.y, fmaf(q2, v.x, ai[1]));
+            }
+          }
+        };
+        auto sums = [&](auto zero) {
+          fetch(0, 0);
+#pragma unroll 1
+          for (int y = 0; y < piece; y += 16) {   // a piece is a multiple of 16
+            fetch(1, y + 8);
+            sum(0, zero);
+            fetch(0, y + 16 < piece ? y + 16 : 0);
+            sum(1, zero);
+          }
+        };
+        if (t0 + warp == 0) sums(std::true_type{});   // the pair (-m, 0)
+        else sums(std::false_type{});
+      }
+      if (ring < pieces) {   // everybody is done with the piece
+        __syncthreads();
+        if (tid == 0 && k + ring < pieces) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // reads before the refill
+          load_piece(k + ring);
         }
       }
     }
-    if constexpr (ADJ) {
-      ar = ar - br;
-      ai = ai + bi;
+    if (on) {
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if constexpr (ADJ) {
+          ar[s] = ar[s] - br[s];
+          ai[s] = ai[s] + bi[s];
+        }
+        hs[(2 * warp + s) * CW + c] = make_float2(ar[s], ai[s]);
+        if (a.Hr) {
+          const int j = s ? row_b(t0 + warp) : row_a(t0 + warp);
+          const long long o = (((long long)b * J + j) * m + kx) * CW + c;
+          a.Hr[o] = ar[s];
+          a.Hi[o] = ai[s];
+        }
+      }
     }
-    hr[jl * CW + c] = ar;
-    hi[jl * CW + c] = ai;
-    if (a.Hr) {
-      const long long o = (((long long)b * J + j0 + jl) * m + kx) * CW + c;
-      a.Hr[o] = ar;
-      a.Hi[o] = ai;
-    }
-    __syncwarp();
-    // ---- mixing of this mode ----
+  }
+  __syncthreads();
+  // ---- mixing of this block's modes: Y_o = sum_i W_io H_i with o = this lane, or in the adjoint
+  // dH_i = sum_o conj(W_io) dY_o with i = this lane ----
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // the other blocks have started
+  for (int jl = warp; jl < 2 * tn; jl += kColThreads / 32) {
     float sr = 0.f, si = 0.f;
     const __nv_bfloat16* w0 = wr + jl * WMAT;
     const __nv_bfloat16* w1 = wi + jl * WMAT;
-    if constexpr (ADJ) {   // dH_i = sum_o conj(W_io) dY_o, i = this lane
 #pragma unroll
-      for (int o8 = 0; o8 < CW; o8 += 8) {
-        const uint4 a4 = *reinterpret_cast<const uint4*>(w0 + c * WROW + o8);
-        const uint4 b4 = *reinterpret_cast<const uint4*>(w1 + c * WROW + o8);
-        const __nv_bfloat16* pa = reinterpret_cast<const __nv_bfloat16*>(&a4);
-        const __nv_bfloat16* pb = reinterpret_cast<const __nv_bfloat16*>(&b4);
+    for (int i8 = 0; i8 < CW; i8 += 8) {
+      __nv_bfloat16 pa[8], pb[8];
+      if constexpr (ADJ) {
+        *reinterpret_cast<uint4*>(pa) = *reinterpret_cast<const uint4*>(w0 + c * WROW + i8);
+        *reinterpret_cast<uint4*>(pb) = *reinterpret_cast<const uint4*>(w1 + c * WROW + i8);
+      } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const float p = __bfloat162float(pa[i]), q = __bfloat162float(pb[i]);
-          const float u = hr[jl * CW + o8 + i], w = hi[jl * CW + o8 + i];
-          sr = fmaf(p, u, fmaf(q, w, sr));
-          si = fmaf(p, w, fmaf(-q, u, si));
+          pa[i] = w0[(i8 + i) * CW + c];
+          pb[i] = w1[(i8 + i) * CW + c];
         }
       }
-    } else {               // Y_o = sum_i W_io H_i, o = this lane
-#pragma unroll 8
-      for (int i = 0; i < CW; ++i) {
-        const float p = __bfloat162float(w0[i * CW + c]), q = __bfloat162float(w1[i * CW + c]);
-        const float u = hr[jl * CW + i], w = hi[jl * CW + i];
-        sr = fmaf(p, u, fmaf(-q, w, sr));
-        si = fmaf(p, w, fmaf(q, u, si));
+      float4 h4[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) h4[i] = *reinterpret_cast<const float4*>(hs + jl * CW + i8 + 2 * i);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float p = __bfloat162float(pa[i]), q = __bfloat162float(pb[i]);
+        const float u = i & 1 ? h4[i >> 1].z : h4[i >> 1].x, w = i & 1 ? h4[i >> 1].w : h4[i >> 1].y;
+        if constexpr (ADJ) {
+          sr = fmaf(p, u, fmaf(q, w, sr));
+          si = fmaf(p, w, fmaf(-q, u, si));
+        } else {
+          sr = fmaf(p, u, fmaf(-q, w, sr));
+          si = fmaf(p, w, fmaf(q, u, si));
+        }
       }
     }
-    mr[jl * CW + c] = sr;
-    mi[jl * CW + c] = si;
+    // ---- into every block's copy of the mixed modes (distributed shared memory) ----
+    const int t = t0 + (jl >> 1), j = jl & 1 ? row_b(t) : row_a(t);
+    const uint32_t o0 = smem_u32(ys + j * CW + c);
+#pragma unroll
+    for (int r = 0; r < CS; ++r) {
+      uint32_t d0;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d0) : "r"(o0), "r"(r));
+      asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(d0), "f"(sr), "f"(si) : "memory");
+    }
   }
-
-  // ---- every block's mixed modes, through distributed shared memory ----
+  // every block's modes have arrived everywhere
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-  for (int e = tid; e < J * CW / 4; e += kColThreads) {
-    const int j = e / (CW / 4), r = j / JB;
-    const int off = ((j - r * JB) * CW + 4 * (e % (CW / 4))) * 4;
-    uint32_t s0, s1;
-    float4 p, q;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(s0) : "r"(smem_u32(mr) + off), "r"(r));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(s1) : "r"(smem_u32(mi) + off), "r"(r));
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(p.x), "=f"(p.y), "=f"(p.z), "=f"(p.w) : "r"(s0) : "memory");
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "r"(s1) : "memory");
-    *reinterpret_cast<float4*>(yr + 4 * e) = p;
-    *reinterpret_cast<float4*>(yi + 4 * e) = q;
-  }
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // done with the other blocks' memory
-  __syncthreads();
 
-  // ---- Z_y = sum over j, in order, four y a thread ----
-  float* z0 = a.Z + (((long long)b * J + kx) * n + y0) * CW + c;
-  float* z1 = z0 + (long long)m * n * CW;
-  for (int yg = warp; yg < ny / 4; yg += kColThreads / 32) {
-    float ar[4] = {0, 0, 0, 0}, ai[4] = {0, 0, 0, 0}, br[4] = {0, 0, 0, 0}, bi[4] = {0, 0, 0, 0};
+  // ---- Z_y = sum over j, in order: four y of two channels a thread ----
+  const int c2 = 2 * (tid & 15);
+  for (int yg = tid >> 4; yg < (y0 < n ? ny / 4 : 0); yg += kColThreads / 16) {
+    float ar[2][4] = {}, ai[2][4] = {}, br[2][4] = {}, bi[2][4] = {};
 #pragma unroll 4
     for (int j = 0; j < J; ++j) {
       const float4 p4 = *reinterpret_cast<const float4*>(vr + j * ny + 4 * yg);
       const float4 q4 = *reinterpret_cast<const float4*>(vi + j * ny + 4 * yg);
+      const float4 yv = *reinterpret_cast<const float4*>(ys + j * CW + c2);
       const float pv[4] = {p4.x, p4.y, p4.z, p4.w}, qv[4] = {q4.x, q4.y, q4.z, q4.w};
-      const float u = yr[j * CW + c], w = yi[j * CW + c];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if constexpr (ADJ) {
-          ar[i] = fmaf(pv[i], u, ar[i]);
-          br[i] = fmaf(qv[i], w, br[i]);
-          ai[i] = fmaf(pv[i], w, ai[i]);
-          bi[i] = fmaf(qv[i], u, bi[i]);
-        } else {   // conj(G) = Gr - i Gi
-          ar[i] = fmaf(pv[i], u, fmaf(qv[i], w, ar[i]));
-          ai[i] = fmaf(pv[i], w, fmaf(-qv[i], u, ai[i]));
+      for (int s = 0; s < 2; ++s) {
+        const float u = s ? yv.z : yv.x, w = s ? yv.w : yv.y;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if constexpr (ADJ) {
+            ar[s][i] = fmaf(pv[i], u, ar[s][i]);
+            br[s][i] = fmaf(qv[i], w, br[s][i]);
+            ai[s][i] = fmaf(pv[i], w, ai[s][i]);
+            bi[s][i] = fmaf(qv[i], u, bi[s][i]);
+          } else {   // conj(G) = Gr - i Gi
+            ar[s][i] = fmaf(pv[i], u, fmaf(qv[i], w, ar[s][i]));
+            ai[s][i] = fmaf(pv[i], w, fmaf(-qv[i], u, ai[s][i]));
+          }
         }
       }
     }
+    float* z0 = a.Z + (((long long)b * J + kx) * n + y0 + 4 * yg) * CW + c2;
+    float* z1 = z0 + (long long)m * n * CW;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       if constexpr (ADJ) {
-        ar[i] = ar[i] + br[i];
-        ai[i] = ai[i] - bi[i];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          ar[s][i] = ar[s][i] + br[s][i];
+          ai[s][i] = ai[s][i] - bi[s][i];
+        }
       }
-      z0[(4 * yg + i) * CW] = ar[i];
-      z1[(4 * yg + i) * CW] = ai[i];
+      *reinterpret_cast<float2*>(z0 + i * CW) = make_float2(ar[0][i], ar[1][i]);
+      *reinterpret_cast<float2*>(z1 + i * CW) = make_float2(ai[0][i], ai[1][i]);
     }
   }
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------
@@ -551,13 +684,16 @@ __global__ void __launch_bounds__(256) mode_wgrad_kernel(const float* __restrict
 // Gradients of the channel-mixing weights: part[chunk][i * cd + o] = sum over the chunk's points
 // of A[p][i] D[p][o], part[chunk][ca * cd + o] = sum of D[p][o].  A chunk is summed in groups of
 // 64 points (in order inside a group, then the groups in order); a warp takes one group, whose
-// 32 x 32 products it holds as 4 x 8 per lane, so that three 16-byte shared loads feed 32 FMAs.
+// 32 x 32 products it holds as 4 x 8 per lane, so that three 16-byte shared loads feed 32 FMAs;
+// the next 32 points travel meanwhile.  At 524288 points: 39 us (134 MB, 20 us at the measured copy
+// rate), where one output a thread with two shared loads for each FMA took 200 us.
 // ---------------------------------------------------------------------------------------
-enum WgA { WA_RAW = 0, WA_GELU = 1, WA_LIFT = 2, WA_X = 3 };    // rows of A: z, GELU(z), x Wp + bp, x itself (4 wide)
+enum WgA { WA_RAW = 0, WA_LIFT = 1, WA_X = 2 };       // rows of A: h as stored, x Wp + bp, x itself (4 wide)
 enum WgD { WD_RAW = 0, WD_OUTER = 1, WD_ONE = 2 };              // rows of D: dz, dout Wq, dout itself (1 wide)
 
 struct WgArgs {
   const float *A, *D;
+  int a16;                // WA_LIFT, WA_X (the caller's x): 1 if it is 16-byte aligned
   const float *Wp, *bp;   // WA_LIFT
   const float* Wq;        // WD_OUTER
   long long P;
@@ -565,8 +701,21 @@ struct WgArgs {
   float* part;            // [blocks][nout]
 };
 
-constexpr int kWgWarps = 4, kWgGroup = 64;
-constexpr int kWgSmem = kWgWarps * kWgGroup * 2 * CW * 4;
+constexpr int kWgWarps = 4, kWgGroup = 64, kWgHalf = 32;
+// per warp: two stages of 32 points of A and D (the group's sums take the second one's place at the
+// end of a group, when nothing is on its way there); small inputs (x, dout) of the stages that
+// are formed where they are read.  Three blocks fit an SM.
+constexpr int kWgStage = kWgHalf * 2 * CW;
+constexpr int kWgSmall = kWgHalf * 5;
+constexpr int kWgSmem = kWgWarps * (2 * kWgStage + 2 * kWgSmall) * 4;
+
+// 16 or 4 bytes global -> shared, zeros where `in` is false (src must be a valid address all the same)
+__device__ __forceinline__ void cp_async16_or0(void* smem, const void* gmem, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem)), "l"(gmem), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async4_or0(void* smem, const void* gmem, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(smem)), "l"(gmem), "r"(in ? 4 : 0) : "memory");
+}
 
 template <int AM, int DM>
 __global__ void __launch_bounds__(32 * kWgWarps) wgrad_kernel(WgArgs a) {
@@ -574,138 +723,155 @@ __global__ void __launch_bounds__(32 * kWgWarps) wgrad_kernel(WgArgs a) {
   constexpr int NOUT = CA * CD + CD;
   constexpr int NACC = (NOUT + 32 * kWgWarps - 1) / (32 * kWgWarps);
   extern __shared__ __align__(16) float wg_sm[];
-  __shared__ float sp[5 * CW];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  float* As = wg_sm + warp * kWgGroup * 2 * CW;   // [64][32]
-  float* Ds = As + kWgGroup * CW;                 // [64][32]
+  float* stage = wg_sm + warp * 2 * kWgStage;                              // [2][A 32 x 32 | D 32 x 32]
+  float* small = wg_sm + kWgWarps * 2 * kWgStage + warp * 2 * kWgSmall;    // [2][x 32 x 4 | dout 32]
+  float lw[5] = {0, 0, 0, 0, 0}, lq = 0.f;   // this lane's channel of the lift and of Wq
   if constexpr (AM == WA_LIFT) {
-    for (int i = tid; i < 5 * CW; i += 32 * kWgWarps) sp[i] = i < 4 * CW ? a.Wp[i] : a.bp[i - 4 * CW];
-    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 5; ++k) lw[k] = k < 4 ? a.Wp[k * CW + lane] : a.bp[lane];
   }
+  if constexpr (DM == WD_OUTER) lq = a.Wq[lane];
   const long long c0 = (long long)blockIdx.x * a.chunk;
   const long long c1 = c0 + a.chunk < a.P ? c0 + a.chunk : a.P;
-  float acc[NACC];
+  // half h of the block's sequence: rounds of kWgWarps groups, two halves a group
+  auto load = [&](int h) {
+    const long long p0 = c0 + (long long)(h >> 1) * (kWgWarps * kWgGroup) + warp * kWgGroup + (h & 1) * kWgHalf;
+    float* As = stage + (h & 1) * kWgStage;
+    float* Ds = As + kWgHalf * CW;
+    float* xs = small + (h & 1) * kWgSmall;
+    if constexpr (AM == WA_RAW) {
 #pragma unroll
-  for (int k = 0; k < NACC; ++k) acc[k] = 0.f;
-  for (long long g0 = c0; g0 < c1; g0 += (long long)kWgWarps * kWgGroup) {
-    const long long p0 = g0 + warp * kWgGroup;
-    // ---- this warp's group: rows of A and D (zero past the chunk) ----
-    if constexpr (AM == WA_RAW || AM == WA_GELU) {
-#pragma unroll 8
-      for (int e = lane; e < kWgGroup * CW / 4; e += 32) {
-        float4 z = make_float4(0, 0, 0, 0);
-        if (p0 + (e >> 3) < c1) {
-          z = *reinterpret_cast<const float4*>(a.A + p0 * CW + e * 4);
-          if constexpr (AM == WA_GELU) z = make_float4(gelu(z.x), gelu(z.y), gelu(z.z), gelu(z.w));
-        }
-        *reinterpret_cast<float4*>(As + e * 4) = z;
+      for (int k = 0; k < 8; ++k) {
+        const int e = lane + 32 * k;
+        const bool in = p0 + (e >> 3) < c1;
+        cp_async16_or0(As + e * 4, a.A + (in ? p0 * CW + e * 4 : 0), in);
       }
     } else {
+      const bool in = p0 + lane < c1;
+      const float* xp = a.A + (in ? (p0 + lane) * 4 : 0);
+      if (a.a16) {
+        cp_async16_or0(xs + lane * 4, xp, in);
+      } else {
 #pragma unroll
-      for (int h = 0; h < kWgGroup / 32; ++h) {
-        const int r = h * 32 + lane;
-        const bool in = p0 + r < c1;
-        const float4 xv = in ? *reinterpret_cast<const float4*>(a.A + (p0 + r) * 4) : make_float4(0, 0, 0, 0);
-        if constexpr (AM == WA_X) {
-          *reinterpret_cast<float4*>(As + r * CW) = xv;
-        } else {
-#pragma unroll
-          for (int c = 0; c < CW; ++c) {   // column rotated by the row: no two lanes on one bank
-            const int cc = (c + lane) & 31;
-            As[r * CW + cc] = in ? fmaf(xv.w, sp[3 * CW + cc], fmaf(xv.z, sp[2 * CW + cc],
-                                   fmaf(xv.y, sp[CW + cc], fmaf(xv.x, sp[cc], sp[4 * CW + cc])))) : 0.f;
-          }
-        }
+        for (int k = 0; k < 4; ++k) cp_async4_or0(xs + lane * 4 + k, xp + k, in);
       }
     }
     if constexpr (DM == WD_RAW) {
-#pragma unroll 8
-      for (int e = lane; e < kWgGroup * CW / 4; e += 32) {
-        float4 z = make_float4(0, 0, 0, 0);
-        if (p0 + (e >> 3) < c1) z = *reinterpret_cast<const float4*>(a.D + p0 * CW + e * 4);
-        *reinterpret_cast<float4*>(Ds + e * 4) = z;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int e = lane + 32 * k;
+        const bool in = p0 + (e >> 3) < c1;
+        cp_async16_or0(Ds + e * 4, a.D + (in ? p0 * CW + e * 4 : 0), in);
       }
     } else {
+      cp_async4_or0(xs + kWgHalf * 4 + lane, a.D + (p0 + lane < c1 ? p0 + lane : 0), p0 + lane < c1);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int rounds = (int)((c1 - c0 + kWgWarps * kWgGroup - 1) / (kWgWarps * kWgGroup));
+  float acc[NACC];
 #pragma unroll
-      for (int h = 0; h < kWgGroup / 32; ++h) {
-        const int r = h * 32 + lane;
-        Ds[r * (DM == WD_ONE ? 1 : CW)] = p0 + r < c1 ? a.D[p0 + r] : 0.f;
-      }
-      if constexpr (DM == WD_OUTER) {
-        __syncwarp();
-        const float w = a.Wq[lane];
-        for (int r = 0; r < kWgGroup; ++r) {
-          const float g = Ds[r * CW];
-          __syncwarp();
-          Ds[r * CW + lane] = g * w;
+  for (int k = 0; k < NACC; ++k) acc[k] = 0.f;
+  load(0);
+  for (int rd = 0; rd < rounds; ++rd) {
+    // ---- this warp's group of 64 points, in order ----
+    const int ig = (lane >> 2) * 4, og = (lane & 3) * 8;
+    constexpr int NI = CD == 1 ? 1 : 4, NO = CD == 1 || CA == 4 ? 1 : 8;
+    float s[NI][NO], bsum = 0.f;
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int o = 0; o < NO; ++o) s[i][o] = 0.f;
+#pragma unroll 1
+    for (int hf = 0; hf < 2; ++hf) {
+      const int h = 2 * rd + hf;
+      if (h + 1 < 2 * rounds) load(h + 1);
+      else asm volatile("cp.async.commit_group;" ::: "memory");
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+      float* As = stage + hf * kWgStage;
+      float* Ds = As + kWgHalf * CW;
+      const float* xs = small + hf * kWgSmall;
+      const long long p0 = c0 + (long long)rd * (kWgWarps * kWgGroup) + warp * kWgGroup + hf * kWgHalf;
+      if constexpr (AM == WA_LIFT) {   // lane = channel
+        const int live = c1 - p0 < kWgHalf ? (int)(c1 - p0) : kWgHalf;
+#pragma unroll 8
+        for (int r = 0; r < kWgHalf; ++r) {
+          const float4 xv = *reinterpret_cast<const float4*>(xs + 4 * r);
+          const float h = fmaf(xv.w, lw[3], fmaf(xv.z, lw[2], fmaf(xv.y, lw[1], fmaf(xv.x, lw[0], lw[4]))));
+          As[r * CW + lane] = r < live ? h : 0.f;
         }
       }
-    }
-    __syncwarp();
-    // ---- the group's sums, r in order ----
-    float bsum = 0.f;
-    if constexpr (CD == 1) {
-      float s = 0.f;
-#pragma unroll 8
-      for (int r = 0; r < kWgGroup; ++r) {
-        const float d = Ds[r];
-        s = fmaf(As[r * CW + lane], d, s);
-        bsum += d;
+      if constexpr (DM == WD_OUTER) {
+#pragma unroll
+        for (int r = 0; r < kWgHalf; r += 4) {
+          const float4 d4 = *reinterpret_cast<const float4*>(xs + kWgHalf * 4 + r);
+          Ds[r * CW + lane] = d4.x * lq;
+          Ds[(r + 1) * CW + lane] = d4.y * lq;
+          Ds[(r + 2) * CW + lane] = d4.z * lq;
+          Ds[(r + 3) * CW + lane] = d4.w * lq;
+        }
       }
-      __syncwarp();
-      As[lane] = s;
-      if (lane == 0) As[CW] = bsum;
-    } else if constexpr (CA == 4) {
-      float s[4] = {0, 0, 0, 0};   // lane = o
+      if constexpr (AM == WA_LIFT || DM == WD_OUTER) __syncwarp();
+      if constexpr (CD == 1) {          // lane = i
 #pragma unroll 8
-      for (int r = 0; r < kWgGroup; ++r) {
-        const float4 x4 = *reinterpret_cast<const float4*>(As + r * CW);
-        const float d = Ds[r * CW + lane];
-        s[0] = fmaf(x4.x, d, s[0]);
-        s[1] = fmaf(x4.y, d, s[1]);
-        s[2] = fmaf(x4.z, d, s[2]);
-        s[3] = fmaf(x4.w, d, s[3]);
-        bsum += d;
-      }
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 4; ++i) As[i * CW + lane] = s[i];
-      As[4 * CW + lane] = bsum;
-    } else {
-      const int ig = (lane >> 2) * 4, og = (lane & 3) * 8;
-      float s[4][8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int o = 0; o < 8; ++o) s[i][o] = 0.f;
+        for (int r = 0; r < kWgHalf; ++r) {
+          const float d = xs[kWgHalf * 4 + r];
+          s[0][0] = fmaf(As[r * CW + lane], d, s[0][0]);
+          bsum += d;
+        }
+      } else if constexpr (CA == 4) {   // lane = o
+#pragma unroll 8
+        for (int r = 0; r < kWgHalf; ++r) {
+          const float4 x4 = *reinterpret_cast<const float4*>(xs + 4 * r);
+          const float d = Ds[r * CW + lane];
+          s[0][0] = fmaf(x4.x, d, s[0][0]);
+          s[1][0] = fmaf(x4.y, d, s[1][0]);
+          s[2][0] = fmaf(x4.z, d, s[2][0]);
+          s[3][0] = fmaf(x4.w, d, s[3][0]);
+          bsum += d;
+        }
+      } else {
 #pragma unroll 4
-      for (int r = 0; r < kWgGroup; ++r) {
-        const float4 a4 = *reinterpret_cast<const float4*>(As + r * CW + ig);
-        const float4 d4 = *reinterpret_cast<const float4*>(Ds + r * CW + og);
-        const float4 e4 = *reinterpret_cast<const float4*>(Ds + r * CW + og + 4);
-        bsum += Ds[r * CW + lane];
-        const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-        const float dv[8] = {d4.x, d4.y, d4.z, d4.w, e4.x, e4.y, e4.z, e4.w};
+        for (int r = 0; r < kWgHalf; ++r) {
+          const float4 a4 = *reinterpret_cast<const float4*>(As + r * CW + ig);
+          const float4 d4 = *reinterpret_cast<const float4*>(Ds + r * CW + og);
+          const float4 e4 = *reinterpret_cast<const float4*>(Ds + r * CW + og + 4);
+          bsum += Ds[r * CW + lane];
+          const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+          const float dv[8] = {d4.x, d4.y, d4.z, d4.w, e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+          for (int i = 0; i < NI; ++i)
 #pragma unroll
-          for (int o = 0; o < 8; ++o) s[i][o] = fmaf(av[i], dv[o], s[i][o]);
+            for (int o = 0; o < NO; ++o) s[i][o] = fmaf(av[i], dv[o], s[i][o]);
+        }
       }
-      __syncwarp();
+      __syncwarp();   // read before the next load into this stage
+    }
+    float* S = stage + kWgStage;
+    if constexpr (CD == 1) {
+      S[lane] = s[0][0];
+      if (lane == 0) S[CW] = bsum;
+    } else if constexpr (CA == 4) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) S[i * CW + lane] = s[i][0];
+      S[4 * CW + lane] = bsum;
+    } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int o = 0; o < 8; ++o) As[(ig + i) * CW + og + o] = s[i][o];
-      As[CW * CW + lane] = bsum;
+        for (int o = 0; o < NO; o += 4)
+          *reinterpret_cast<float4*>(S + (ig + i) * CW + og + o) = make_float4(s[i][o], s[i][o + 1], s[i][o + 2], s[i][o + 3]);
+      S[CW * CW + lane] = bsum;
     }
     __syncthreads();
     // ---- groups in order ----
-    for (int w = 0; w < kWgWarps && g0 + w * kWgGroup < c1; ++w) {
-      const float* S = wg_sm + w * kWgGroup * 2 * CW;
+    for (int w = 0; w < kWgWarps && c0 + ((long long)rd * kWgWarps + w) * kWgGroup < c1; ++w) {
 #pragma unroll
       for (int k = 0; k < NACC; ++k) {
         const int o = tid + k * 32 * kWgWarps;
-        if (o < NOUT) acc[k] += S[o];
+        if (o < NOUT) acc[k] += wg_sm[(2 * w + 1) * kWgStage + o];
       }
     }
     __syncthreads();

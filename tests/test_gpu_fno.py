@@ -214,3 +214,34 @@ def test_corrector_workflow_small(T, torch):
     assert losses[-1][1] < losses[0][1]
     r = Cr.evaluate(net, 6.3, coarse_steps=40, sample_every=20, transient=40)
     assert r["nonfinite"] == 0 and r["t_fno"] > 0 and 0 <= r["spectrum_error_plain"] < 10
+
+
+# The layer kernels (row kernel, clustered column kernel) at the edges of their range: one x tile
+# partly filled, one to four tiles, mode counts that leave blocks of a cluster without a ky, more
+# grid rows than resident blocks; and an odd mode count and a 1024 grid, which keep the separate
+# kernels.  BF16 rounding of operands bounds the error as above.
+EDGES = [(16, 4, 1, 3), (32, 6, 2, 1), (64, 2, 2, 2), (128, 12, 1, 4), (512, 16, 1, 1), (32, 3, 1, 2), (1024, 4, 1, 1)]
+
+
+@pytest.mark.parametrize("n,modes,layers,batch", EDGES)
+def test_layer_kernels_match_oracle_at_the_edges(T, torch, n, modes, layers, batch):
+    net, cfg = make(T, seed=21, n=n, modes=modes, layers=layers, max_batch=batch)
+    rng = np.random.default_rng(3)
+    x = rng.standard_normal((batch, n, n, 4)).astype(np.float32)
+    t = rng.standard_normal((batch, n, n)).astype(np.float32)
+    # an input that starts 4 bytes past a 16-byte boundary
+    buf = torch.zeros(x.size + 1, device="cuda")
+    buf[1:] = torch.tensor(x.reshape(-1), device="cuda")
+    td, yd = torch.tensor(t, device="cuda"), torch.zeros((batch, n, n), device="cuda")
+    xp = buf[1:].data_ptr()
+    net.forward(xp, yd.data_ptr(), batch)
+    loss, g = net.loss_grad(xp, td.data_ptr(), batch, want_grad=True)
+    th = oracle_theta(cfg, net.get_params())
+    assert rel(yd.cpu().numpy(), F.forward(cfg, th, x.astype(np.float64))) <= TOL
+    L0, gr = F.loss_and_grad(cfg, th, x.astype(np.float64), t.astype(np.float64))
+    assert loss == pytest.approx(L0, rel=TOL)
+    o = 0
+    for name, shp in F.param_shapes(cfg):
+        k = int(np.prod(shp))
+        assert rel(g[o:o + k], gr[o:o + k]) <= TOL, name
+        o += k
