@@ -47,6 +47,21 @@ template <typename T>
 __device__ __forceinline__ cplx<T> operator+(cplx<T> a, cplx<T> b) { return mk(a.x + b.x, a.y + b.y); }
 template <typename T>
 __device__ __forceinline__ cplx<T> operator-(cplx<T> a, cplx<T> b) { return mk(a.x - b.x, a.y - b.y); }
+// Float: both parts in one packed instruction (the same roundings).  The packed add takes the FP32
+// pipe as long as the two it replaces, but one issue slot instead of two, and the transform
+// passes of the larger grids are bound by issue.
+__device__ __forceinline__ cplx<float> operator+(cplx<float> a, cplx<float> b) {
+  cplx<float> r;
+  asm("{\n.reg .b64 a, b, c;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 c, a, b;\nmov.b64 {%0, %1}, c;\n}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ cplx<float> operator-(cplx<float> a, cplx<float> b) {
+  cplx<float> r;
+  asm("{\n.reg .b64 a, b, c;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nsub.rn.f32x2 c, a, b;\nmov.b64 {%0, %1}, c;\n}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
 template <typename T>
 __device__ __forceinline__ cplx<T> operator*(cplx<T> a, T s) { return mk(a.x * s, a.y * s); }
 template <typename T>
@@ -102,8 +117,9 @@ __device__ __forceinline__ cplx<T> rot16(cplx<T> d, int j) {
 }
 
 // In-register R-point DFT (R <= 16), sign DIR.  Radix-2 decimation in frequency: on exit
-// v[bitrev(k)] holds X[k].
-template <typename T, int R, int DIR>
+// v[bitrev(k)] holds X[k].  BAND: v[i] is zero for R/4 < i < 3R/4 (and may hold anything there),
+// so all but one of the first layer's butterflies copy.
+template <typename T, int R, int DIR, bool BAND = false>
 __device__ __forceinline__ void dft_reg(cplx<T>* v) {
 #pragma unroll
   for (int half = R / 2; half >= 1; half >>= 1) {
@@ -113,8 +129,15 @@ __device__ __forceinline__ void dft_reg(cplx<T>* v) {
       for (int i = 0; i < half; ++i) {
         const cplx<T> a = v[blk + i];
         const cplx<T> b = v[blk + i + half];
-        v[blk + i] = a + b;
-        v[blk + i + half] = rot16<T, DIR>(a - b, i * (16 / (2 * half)));
+        if (BAND && half == R / 2 && i < R / 4) {          // b = 0
+          v[i + half] = rot16<T, DIR>(a, i * (16 / (2 * half)));
+        } else if (BAND && half == R / 2 && i > R / 4) {   // a = 0
+          v[i] = b;
+          v[i + half] = rot16<T, DIR>(mk<T>(-b.x, -b.y), i * (16 / (2 * half)));
+        } else {
+          v[blk + i] = a + b;
+          v[blk + i + half] = rot16<T, DIR>(a - b, i * (16 / (2 * half)));
+        }
       }
     }
   }
@@ -268,18 +291,27 @@ __device__ __forceinline__ int handoff_slot(int i) {
   else return (i & ~15) | ((i + ((i >> 3) & 8)) & 15);
 }
 
+// Band-limited transforms: inputs (BAND_IN) or outputs (BAND_OUT) m with L/4 < m < 3L/4 are zero or
+// not wanted.  The first stage then loads only the elements inside the band, the last one
+// computes and stores only those (the buffer keeps what it held elsewhere).
+enum Band { BAND_NONE = 0, BAND_IN = 1, BAND_OUT = 2 };
+
 // One Stockham stage of radix R on a length-L transform at buf (padded), current
 // sub-transform length Ns.  j: this thread's index among the L/PE owners.  In the first
-// stage (Ns = 1) an input functor ld(bi, m) may supply element m of transform bi instead of
-// the buffer (fusing the caller's pre-pass into the stage); that stage then reads nothing
-// from the buffer, so it needs no barrier between its loads and its stores.
-template <typename T, int L, int PE, int R, int Ns, int DIR, int PS, int TWN, int NT, typename LD>
+// stage (Ns = 1) an input functor ld(bi, m, upper) may supply element m of transform bi instead
+// of the buffer (fusing the caller's pre-pass into the stage; upper, a compile-time constant,
+// says m >= L/2); that stage then reads nothing from the buffer, so it needs no barrier between
+// its loads and its stores.
+template <typename T, int L, int PE, int R, int Ns, int DIR, int PS, int TWN, int NT, int BAND, typename LD>
 __device__ __forceinline__ void stockham_stage(cplx<T>* buf, int j, bool active,
                                                const TwTab<T, TWN>& tw, const cplx<T>* stab,
                                                int bi, const LD& ld) {
   constexpr int TT = L / PE;
   constexpr int NB = PE / R;
   constexpr bool FUSED = Ns == 1 && !std::is_same<LD, NoLoad>::value;
+  constexpr bool IN = BAND == BAND_IN && FUSED && R >= 4;
+  constexpr bool OUT = BAND == BAND_OUT && Ns * R == L && R >= 4;   // r Ns + q is the output's index
+  static_assert(BAND != BAND_IN || Ns > 1 || IN, "a band-limited input needs an input functor and radix >= 4");
   // Padded index of i + d: when adding d cannot carry out of the low PS bits of i (d a
   // multiple of the padding interval, or every index below one interval), padi(i + d) =
   // padi(i) + d + (d >> PS), so one padded base and compile-time offsets serve all of a
@@ -303,7 +335,17 @@ __device__ __forceinline__ void stockham_stage(cplx<T>* buf, int j, bool active,
       const int q = j + b * TT;
       if constexpr (FUSED) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[b][r] = ld(bi, q + r * SL);
+        for (int r = 0; r < R; ++r) {
+          if (IN && r > R / 4 && r < 3 * R / 4) continue;   // outside the band
+          if (IN && r == R / 4) {                           // only its first element is inside
+            v[b][r] = mk<T>(0, 0);
+            if (q == 0) v[b][r] = ld(bi, q + r * SL, std::false_type{});
+          } else if (r < R / 2) {
+            v[b][r] = ld(bi, q + r * SL, std::false_type{});
+          } else {
+            v[b][r] = ld(bi, q + r * SL, std::true_type{});
+          }
+        }
       } else if constexpr (ROT_IN) {
 #pragma unroll
         for (int r = 0; r < R; ++r) v[b][r] = buf[handoff_slot<PE>(q + r * SL)];
@@ -338,7 +380,7 @@ __device__ __forceinline__ void stockham_stage(cplx<T>* buf, int j, bool active,
           for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], twiddle<T, DIR>(tw, r * k * stride));
         }
       }
-      dft_reg<T, R, DIR>(v[b]);
+      dft_reg<T, R, DIR, IN>(v[b]);
       const int base = (q - k) * R + k;
       if constexpr (ROT_OUT) {
 #pragma unroll
@@ -346,34 +388,37 @@ __device__ __forceinline__ void stockham_stage(cplx<T>* buf, int j, bool active,
       } else if constexpr (ST_OFF) {
         cplx<T>* p0 = buf + padi<PS>(base);
 #pragma unroll
-        for (int r = 0; r < R; ++r) p0[r * Ns + ((r * Ns) >> PS)] = v[b][bitrev<R>(r)];
+        for (int r = 0; r < R; ++r)
+          if (!OUT || r <= R / 4 || r >= 3 * R / 4) p0[r * Ns + ((r * Ns) >> PS)] = v[b][bitrev<R>(r)];
       } else {
 #pragma unroll
-        for (int r = 0; r < R; ++r) buf[padi<PS>(base + r * Ns)] = v[b][bitrev<R>(r)];
+        for (int r = 0; r < R; ++r)
+          if (!OUT || r <= R / 4 || r >= 3 * R / 4) buf[padi<PS>(base + r * Ns)] = v[b][bitrev<R>(r)];
       }
     }
   }
   stage_sync<TT, NT>();
 }
 
-template <typename T, int L, int PE, int Ns, int DIR, int PS, int TWN, int NT, typename LD>
+template <typename T, int L, int PE, int Ns, int DIR, int PS, int TWN, int NT, int BAND, typename LD>
 __device__ __forceinline__ void stockham_all(cplx<T>* buf, int j, bool active,
                                              const TwTab<T, TWN>& tw, const cplx<T>* stab,
                                              int bi, const LD& ld) {
   if constexpr (Ns < L) {
     constexpr int R = (L / Ns < PE) ? (L / Ns) : PE;
-    stockham_stage<T, L, PE, R, Ns, DIR, PS, TWN, NT>(buf, j, active, tw, stab, bi, ld);
-    stockham_all<T, L, PE, Ns * R, DIR, PS, TWN, NT>(buf, j, active, tw, stab, bi, NoLoad{});
+    stockham_stage<T, L, PE, R, Ns, DIR, PS, TWN, NT, BAND>(buf, j, active, tw, stab, bi, ld);
+    stockham_all<T, L, PE, Ns * R, DIR, PS, TWN, NT, BAND>(buf, j, active, tw, stab, bi, NoLoad{});
   }
 }
 
 // B transforms of length L laid out at sm + b * STRIDE (padded; STRIDE = 0 means the padded
 // length), all threads of the block participate (NT threads).  TWN: length of the twiddle
 // table (a multiple of L); stab: this length's per-stage tables (ignored when unused);
-// ld: optional input functor ld(b, m) -> element m of transform b (see stockham_stage).
+// ld: optional input functor ld(b, m, upper) -> element m of transform b (see stockham_stage);
+// BAND: inputs or outputs limited to a band (see Band).
 // Starts with a block barrier and ends with one (the stage barriers in between are warp
 // barriers when every transform lies inside one warp).
-template <typename T, int L, int PE, int DIR, int NT, int TWN, int STRIDE = 0, typename LD = NoLoad>
+template <typename T, int L, int PE, int DIR, int NT, int TWN, int STRIDE = 0, int BAND = BAND_NONE, typename LD = NoLoad>
 __device__ __forceinline__ void fft_batch(cplx<T>* sm, int B, const TwTab<T, TWN>& tw, const cplx<T>* stab,
                                           const LD& ld = LD{}) {
   constexpr int PS = pad_shift<T>();
@@ -387,7 +432,7 @@ __device__ __forceinline__ void fft_batch(cplx<T>* sm, int B, const TwTab<T, TWN
   for (int c0 = 0; c0 < B; c0 += PER) {
     const int b = c0 + slot;
     const bool active = b < B;
-    stockham_all<T, L, PE, 1, DIR, PS, TWN, NT>(sm + (active ? b : 0) * LP, j, active, tw, stab, b, ld);
+    stockham_all<T, L, PE, 1, DIR, PS, TWN, NT, BAND>(sm + (active ? b : 0) * LP, j, active, tw, stab, b, ld);
   }
   if constexpr (TT <= 32 && 32 % TT == 0) block_sync<NT>();
 }

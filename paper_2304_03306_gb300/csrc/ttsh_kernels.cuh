@@ -547,38 +547,36 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
   // ---- inverse row transforms (C2R through an L-point complex transform) ----
   // The twiddle pre-pass that turns the half spectrum X of a real row into the L-point
   // complex input Z[k] = (X[k] + conj X[L-k]) + i conj(W_N^k) (X[k] - conj X[L-k]) is the
-  // input functor of the first transform stage.
+  // input functor of the first transform stage.  With X[m] = 0 for m > M = L/2 only one of the
+  // two is non-zero: Z[k] = X[k] (1 + i conj(W_N^k)) for k < M and conj X[L-k] (1 - i conj(W_N^k))
+  // from there on (at k = M, where both are X[M], the first factor is 0), so an element costs
+  // two shared loads and one complex product.
   if constexpr (FI > 0) {
-    auto load = [&](int bt, int k) -> cplx<T> {
+    auto load = [&](int bt, int k, auto upper) -> cplx<T> {
+      constexpr bool UP = decltype(upper)::value;
       const int f = bt / R, r = bt % R;   // field f (omega, v_x, v_y / the mask) from G plane f
-      cplx<T> X = mk<T>(0, 0), Xm = mk<T>(0, 0);
-      const int km = L - k;
+      const int kk = UP ? L - k : k;      // stored column
+      cplx<T> X;
       if constexpr (Geo::STAGE_G) {
         if constexpr (CL == 1) {
-          const cplx<T>* src = gin + (size_t)f * GPC + r;
-          if (k <= M) X = src[k * Geo::RSP];
-          if (km <= M) Xm = src[km * Geo::RSP];
+          X = gin[(size_t)f * GPC + r + kk * Geo::RSP];
         } else {
           // column kk of this block's row r: slot (kk - o HC, c R + r) of the share of block
           // o that owns it, read through distributed shared memory when o is the other block
-          auto get = [&](int kk) -> cplx<T> {
-            const int o = kk < Geo::HC ? 0 : 1;
-            const int idx = f * GPC + (kk - o * Geo::HC) * Geo::RS + crank * R + r;
-            return o == crank ? gin[idx] : dsmem_ld(dsmem_addr(gin + idx, (unsigned)o), T());
-          };
-          if (k <= M) X = get(k);
-          if (km <= M) Xm = get(km);
+          const int o = kk < Geo::HC ? 0 : 1;
+          const int idx = f * GPC + (kk - o * Geo::HC) * Geo::RS + crank * R + r;
+          X = o == crank ? gin[idx] : dsmem_ld(dsmem_addr(gin + idx, (unsigned)o), T());
         }
       } else {
-        const cplx<T>* src = A.G + (size_t)f * H * N + (y0 + r);
-        if (k <= M) X = src[(size_t)k * N];
-        if (km <= M) Xm = src[(size_t)km * N];
+        X = A.G[(size_t)f * H * N + (y0 + r) + (size_t)kk * N];
       }
-      if (k == 0) X.y = 0;   // the mx = 0 entry of a real row is real
-      const cplx<T> w = conjg(tw.get(k));        // conj(W_N^k)
-      const cplx<T> s = X + conjg(Xm);
-      const cplx<T> d = X - conjg(Xm);
-      return s + mul_i(cmul(w, d));
+      const cplx<T> w = tw.get(k);               // i conj(W) = (W.y, W.x)
+      if constexpr (UP) {
+        return cmul(conjg(X), mk<T>((T)1 - w.y, -w.x));
+      } else {
+        if (k == 0) X.y = 0;   // the mx = 0 entry of a real row is real
+        return cmul(X, mk<T>((T)1 + w.y, w.x));
+      }
     };
     fft_batch<T, L, PE, +1, NT, N, LP>(sm, FI * R, tw, stab, load);
   }
@@ -597,7 +595,7 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
     // F0..F2 at complex slot k of row r (real points 2k in .x, 2k + 1 in .y), computed from
     // omega, v_x, v_y and K as the forward transforms' input; same arithmetic as the
     // in-place loop below
-    auto rhs = [&](int bt, int k) -> cplx<T> {
+    auto rhs = [&](int bt, int k, auto) -> cplx<T> {
       const int f = bt / R, r = bt % R;
       const cplx<T> wz = sm[(0 * R + r) * LP + padi<PS>(k)];
       // the slot's two mask values in one load (the staged rows start 16-byte aligned, N is even)
@@ -712,26 +710,28 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
     griddep_launch();
     // clusters: every block is past its inverse loads, so the shares can take the results
     if constexpr (CL > 1) cluster_sync();
-    for (int e = tid; e < FF * R * H; e += NT) {
-      const int r = e % R;
-      const int t = e / R;
-      const int k = t % H;
-      const int f = t / H;
-      const cplx<T>* row = fw + (f * R + r) * LP;
-      const cplx<T> Zk = row[padi<PS>(k)];
-      const cplx<T> Zm = conjg(row[padi<PS>((L - k) & (L - 1))]);
-      const cplx<T> s = Zk + Zm;
-      const cplx<T> d = Zk - Zm;
-      // X[k] = (Zk + Zm)/2 - (i/2) W^k (Zk - Zm)
-      const cplx<T> X = (s - mul_i(cmul(tw.get(k), d))) * (T)0.5;
-      if constexpr (CL == 1) {
-        A.Rr[((size_t)f * H + k) * N + (y0 + r)] = X;
-      } else {
-        // into slot (column, this block's row) of the share that owns column k
-        const int o = k < Geo::HC ? 0 : 1;
-        const int idx = f * GPC + (k - o * Geo::HC) * Geo::RS + crank * R + r;
-        if (o == crank) gin[idx] = X;
-        else dsmem_st(dsmem_addr(gin + idx, (unsigned)o), X);
+    // Twice the transform of the real row, X[k] = (Zk + Zm) - i W^k (Zk - Zm); the column pass
+    // halves it with its own 1/N.
+#pragma unroll 1
+    for (int f = 0; f < FF; ++f) {
+      for (int e = tid; e < R * H; e += NT) {
+        const int r = e % R, k = e / R;
+        const cplx<T>* row = fw + (f * R + r) * LP;
+        const cplx<T> Zk = row[padi<PS>(k)];
+        const cplx<T> Zm = conjg(row[padi<PS>((L - k) & (L - 1))]);
+        const cplx<T> s = Zk + Zm;
+        const cplx<T> d = Zk - Zm;
+        const cplx<T> w = tw.get(k);
+        const cplx<T> X = mk<T>(fma(w.x, d.y, fma(w.y, d.x, s.x)), fma(-w.x, d.x, fma(w.y, d.y, s.y)));
+        if constexpr (CL == 1) {
+          A.Rr[((size_t)f * H + k) * N + (y0 + r)] = X;
+        } else {
+          // into slot (column, this block's row) of the share that owns column k
+          const int o = k < Geo::HC ? 0 : 1;
+          const int idx = f * GPC + (k - o * Geo::HC) * Geo::RS + crank * R + r;
+          if (o == crank) gin[idx] = X;
+          else dsmem_st(dsmem_addr(gin + idx, (unsigned)o), X);
+        }
       }
     }
     if constexpr (CL > 1) {
@@ -765,6 +765,7 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
   const int tid = threadIdx.x;
   const T kxp = A.dk * (T)kx;
   const T invN = (T)1 / (T)N;
+  const T fwdN = (T)0.5 / (T)N;   // the row pass leaves twice its transform
   constexpr int CB = Geo::CB;
 
   const TwTab<T, N> tw = TwTab<T, N>::fill(reinterpret_cast<cplx<T>*>(smem_raw), A.tw, tid, NT);
@@ -813,11 +814,11 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
       if constexpr (Geo::BULK) {
         const cplx<T>* stg = reinterpret_cast<const cplx<T>*>(smem_raw + Geo::OFF_STG);
         cp_async_wait_all();   // tables, state column
-        fft_batch<T, N, PE, -1, NT, N>(buf, nb, tw, stab, [&](int bt, int m) { return stg[bt * N + m]; });
+        fft_batch<T, N, PE, -1, NT, N, 0, BAND_OUT>(buf, nb, tw, stab, [&](int bt, int m, auto) { return stg[bt * N + m]; });
       } else {
         stage_columns(f0, nb);
         cp_async_wait_all();
-        fft_batch<T, N, PE, -1, NT, N>(buf, nb, tw, stab);
+        fft_batch<T, N, PE, -1, NT, N, 0, BAND_OUT>(buf, nb, tw, stab);
       }
       for (int j = tid; j < NK; j += NT) {
         const int ky = ky_of(j);
@@ -884,18 +885,19 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
           const T om = (T)1 - k2;
           const T E = exp((A.a - om * om) * A.dt);
           const cplx<T> w = ws[j];
-          const cplx<T> r = acc[j] * invN;
+          const cplx<T> r = acc[j] * fwdN;
           wn = (w + r * A.dt) * E;
           if (m2 == 0 || m2 > M * M) wn = mk<T>(0, 0);
+          ws[j].x = m2 > 0 ? invN / k2 : (T)0;   // for the velocities: one division a mode
         } else if constexpr (MODE == COL_PROJECT) {
-          wn = acc[j] * invN;
+          wn = acc[j] * fwdN;
           if (m2 == 0 || m2 > M * M) wn = mk<T>(0, 0);
         } else if constexpr (MODE == COL_ADDW) {
           // correction delta^ = DFT[delta omega] on the 1/2-rule disc, delta^(0) = 0
-          wn = acc[j] * invN;
+          wn = acc[j] * fwdN;
           if (m2 == 0 || m2 > M * M) wn = mk<T>(0, 0);
         } else {   // COL_MASK: keep |m|^2 <= (N/8)^2, fold both 1/N factors of the round trip
-          wn = acc[j] * (invN * invN);
+          wn = acc[j] * (fwdN * invN);
           if (m2 > (N / 8) * (N / 8)) wn = mk<T>(0, 0);
         }
         acc[j] = wn;
@@ -905,9 +907,9 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
           for (int c = 0; c < 2; ++c) {
             T vm;
             if constexpr (MODE == COL_STEP)
-              vm = A.mean_decay * (A.vmean[c] + A.dt * (s0[c] * invN));   // Eq. (avg)
+              vm = A.mean_decay * (A.vmean[c] + A.dt * (s0[c] * fwdN));   // Eq. (avg)
             else
-              vm = s0[c] * invN;                                              // DFT[v](0)
+              vm = s0[c] * fwdN;                                              // DFT[v](0)
             s0[2 + c] = vm;
             A.vmean[c] = vm;
           }
@@ -952,28 +954,33 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
     for (int f0 = 0; f0 < NI; f0 += FB) {
       const int nb = cmin(FB, NI - f0);
       // spectral multipliers of the four fields, applied as the first stage's input functor
-      auto load = [&](int bt, int idx) -> cplx<T> {
+      // (elements outside the 1/2-rule band are left out by the transform's first stage)
+      auto load = [&](int bt, int idx, auto upper) -> cplx<T> {
         const int f = f0 + bt;
-        const int ky = idx <= N / 2 ? idx : idx - N;
-        cplx<T> v = mk<T>(0, 0);
-        if (ky >= -M && ky <= M) {
-          const cplx<T> w = acc[ky >= 0 ? ky : ky + NK];
-          if constexpr (MODE == COL_MASK) {
-            v = w;
+        const int ky = decltype(upper)::value ? idx - N : idx;
+        const int j = decltype(upper)::value ? idx - N + NK : idx;
+        const cplx<T> w = acc[j];
+        if constexpr (MODE == COL_MASK) {
+          return w;
+        } else {
+          if (f == 0) return w * invN;                    // omega
+          const T kyp = A.dk * (T)ky;
+          const int m2 = kx * kx + ky * ky;
+          T inv;
+          if constexpr (MODE == COL_STEP) {
+            inv = ws[j].x;
           } else {
-            const T kyp = A.dk * (T)ky;
-            const int m2 = kx * kx + ky * ky;
             const T k2 = A.dk * A.dk * (T)m2;
-            const T inv = m2 > 0 ? invN / k2 : (T)0;
-            if (f == 0) v = w * invN;                       // omega
-            else if (f == 1) v = mul_i(w) * (kyp * inv);    // v^x = i ky psi^   (stream function)
-            else v = mul_i(w) * (-kxp * inv);               // v^y = -i kx psi^
-            if (m2 == 0 && f >= 1) v = mk<T>(s0[2 + (f - 1)] * invN, (T)0);   // mean flow
+            inv = m2 > 0 ? invN / k2 : (T)0;
           }
+          // v^x = i ky psi^, v^y = -i kx psi^ (stream function); m = 0: the mean flow
+          const T s = (f == 1 ? kyp : -kxp) * inv;
+          cplx<T> v = mul_i(w) * s;
+          if (m2 == 0) v = mk<T>(s0[2 + (f - 1)] * invN, (T)0);
+          return v;
         }
-        return v;
       };
-      fft_batch<T, N, PE, +1, NT, N, 0>(buf, nb, tw, stab, load);
+      fft_batch<T, N, PE, +1, NT, N, 0, BAND_IN>(buf, nb, tw, stab, load);
       if (f0 + nb >= NI) griddep_launch();   // only the last stores are left (see the row pass)
       for (int e = tid; e < nb * N; e += NT) {
         const int b = e / N, y = e % N;
