@@ -463,6 +463,12 @@ __global__ void noise_kernel(double* __restrict__ real, const unsigned char* __r
   }
 }
 
+// The state of a float domain in double: ne values of omega^, then the mean flow.
+__global__ void widen_kernel(const float* __restrict__ w, const float* __restrict__ m, size_t ne, double* __restrict__ out) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < ne + 2; i += (size_t)gridDim.x * blockDim.x)
+    out[i] = (double)(i < ne ? w[i] : m[i - ne]);
+}
+
 __global__ void record_begin_kernel(RecCtl* c, long long base, double* series, long long capacity,
                                     int every, int nblocks, double inv2n2) {
   c->count = 0;
@@ -1140,24 +1146,24 @@ ttsh_status ttsh_get_mask(ttsh_domain* d, double* K) {
 ttsh_status ttsh_get_spectral_state(ttsh_domain* d, double* w_hat, double* v0) {
   if (!d) return fail(TTSH_E_INVALID, "domain is NULL");
   const size_t ne = (size_t)d->H * d->NK * 2;
+  const double *w = static_cast<const double*>(d->dev.what), *m = static_cast<const double*>(d->dev.vmean);
   if (d->elt == sizeof(float)) {
-    std::vector<float> h(ne), m(2);
-    if (w_hat) TTSH_CUDA(cudaMemcpyAsync(h.data(), d->dev.what, ne * sizeof(float), cudaMemcpyDeviceToHost, d->stream), "download state");
-    TTSH_CUDA(cudaMemcpyAsync(m.data(), d->dev.vmean, 2 * sizeof(float), cudaMemcpyDeviceToHost, d->stream), "download mean");
-    ttsh_status st = sync(d, "get_spectral_state");
-    if (st != TTSH_OK) return st;
-    if (w_hat) to_host_double(h, w_hat);
-    if (v0) to_host_double(m, v0);
-  } else {
-    if (w_hat) TTSH_CUDA(cudaMemcpyAsync(w_hat, d->dev.what, ne * sizeof(double), cudaMemcpyDeviceToHost, d->stream), "download state");
-    double m[2];
-    TTSH_CUDA(cudaMemcpyAsync(m, d->dev.vmean, 2 * sizeof(double), cudaMemcpyDeviceToHost, d->stream), "download mean");
-    ttsh_status st = sync(d, "get_spectral_state");
-    if (st != TTSH_OK) return st;
-    if (v0) {
-      v0[0] = m[0];
-      v0[1] = m[1];
-    }
+    // widened on the device (in the staging planes), so that the copy lands in the caller's array
+    const unsigned blocks = (unsigned)std::min<size_t>((ne + 255) / 256, 152 * 16);
+    ttsh::widen_kernel<<<blocks, 256, 0, d->stream>>>(static_cast<const float*>(d->dev.what),
+                                                       static_cast<const float*>(d->dev.vmean), ne, d->dev.real);
+    TTSH_CUDA(cudaGetLastError(), "widen state");
+    w = d->dev.real;
+    m = d->dev.real + ne;
+  }
+  double mean[2];
+  if (w_hat) TTSH_CUDA(cudaMemcpyAsync(w_hat, w, ne * sizeof(double), cudaMemcpyDeviceToHost, d->stream), "download state");
+  TTSH_CUDA(cudaMemcpyAsync(mean, m, sizeof(mean), cudaMemcpyDeviceToHost, d->stream), "download mean");
+  const ttsh_status st = sync(d, "get_spectral_state");
+  if (st != TTSH_OK) return st;
+  if (v0) {
+    v0[0] = mean[0];
+    v0[1] = mean[1];
   }
   return TTSH_OK;
 }

@@ -225,10 +225,10 @@ def ttsh_get_mask(h, n: int):
 
 def ttsh_get_spectral_state(h, n: int):
     M = n // 4
-    buf = np.empty((M + 1, 2 * M + 1, 2))
+    w_hat = np.empty((M + 1, 2 * M + 1), dtype=np.complex128)   # interleaved (re, im), as the library writes it
     v0 = np.empty(2)
-    _check(load_library().ttsh_get_spectral_state(h, _dptr(buf), _dptr(v0)))
-    return buf[..., 0] + 1j * buf[..., 1], v0
+    _check(load_library().ttsh_get_spectral_state(h, _dptr(w_hat), _dptr(v0)))
+    return w_hat, v0
 
 
 def ttsh_set_spectral_state(h, w_hat, v0, n: int):
