@@ -228,7 +228,8 @@ ttsh_status ttsh_set_plan(ttsh_domain* d, int32_t row_variant, int32_t col_varia
 /* Launch mode of the step kernels, a bit set:
  *   bit 0  programmatic dependent launches: a pass may start (copy its twiddle tables and
  *          mask rows) while the previous pass is still running and waits on the device
- *          (griddepcontrol.wait) before it reads anything that pass wrote;
+ *          (griddepcontrol.wait) before it reads anything that pass wrote; on grids up to 512^2
+ *          the library launches its steps so whatever the bit;
  *   bit 1  the row pass loads its G tile with the tensor-memory accelerator (one 2D tile load
  *          per field, completion on an mbarrier with a bounded wait) instead of cp.async,
  *          where the tile allows it (N <= 512, a row segment of R complex values a multiple

@@ -920,6 +920,7 @@ ttsh_status ttsh_create_domain(const uint8_t* mask, const ttsh_params* p, void* 
   v.rec = nullptr;
   v.recctl = nullptr;
   v.pdl = 0;
+  v.whole = 0;
   v.use_tma = 0;
   v.err = reinterpret_cast<int*>(base + d->lay.err);
   v.knaive = reinterpret_cast<unsigned char*>(base + d->lay.knaive);
@@ -1248,11 +1249,10 @@ ttsh_status ttsh_time_kernels(ttsh_domain* d, int32_t iters, double* ms) {
   if (iters < 1 || iters > 1000000) return fail(TTSH_E_INVALID, "iters must be in [1, 1000000]");
   ttsh_status st = save_state(d);
   if (st != TTSH_OK) return st;
-  const int pdl = d->dev.pdl;
-  d->dev.pdl = 0;   // each launch timed whole, with no overlap from the next one
+  d->dev.whole = 1;   // each launch timed whole, with no overlap from the next one
   if ((st = time_launches(d, d->ops.row_step[d->rv].fn, iters, &ms[0])) == TTSH_OK)
     st = time_launches(d, d->ops.col_step[d->cv].fn, iters, &ms[1]);
-  d->dev.pdl = pdl;
+  d->dev.whole = 0;
   if (st != TTSH_OK) return st;
   return restore_state(d);
 }
@@ -1263,26 +1263,33 @@ ttsh_status ttsh_autotune(ttsh_domain* d, int32_t iters, int32_t* plan) {
   if (iters < 1 || iters > 100000) return fail(TTSH_E_INVALID, "iters must be in [1, 100000]");
   ttsh_status st = save_state(d);
   if (st != TTSH_OK) return st;
-  const int pdl0 = d->dev.pdl, tma0 = d->dev.use_tma;
-  d->dev.pdl = 0;   // variants are timed as plain back-to-back launches
+  const int tma0 = d->dev.use_tma;
+  // variants are timed as plain back-to-back launches
+  struct Whole {
+    ttsh::DomainDev& v;
+    explicit Whole(ttsh::DomainDev& dv) : v(dv) { v.whole = 1; }
+    ~Whole() { v.whole = 0; }
+  };
   double best = 1e300;
   int br = 0, bc = 0, btma = 0;
-  for (int i = 0; i < d->ops.n_row_variants; ++i) {
-    for (int tma = 0; tma < 1 + d->ops.row_step[i].tma; ++tma) {   // G tile by cp.async, then by TMA (where the tile allows)
-      d->dev.use_tma = tma;
+  {
+    const Whole whole(d->dev);
+    for (int i = 0; i < d->ops.n_row_variants; ++i) {
+      for (int tma = 0; tma < 1 + d->ops.row_step[i].tma; ++tma) {   // G tile by cp.async, then by TMA (where the tile allows)
+        d->dev.use_tma = tma;
+        double t;
+        if ((st = time_launches(d, d->ops.row_step[i].fn, iters, &t)) != TTSH_OK) return st;
+        if (t < best) { best = t; br = i; btma = tma; }
+      }
+    }
+    d->dev.use_tma = btma;
+    best = 1e300;
+    for (int i = 0; i < d->ops.n_col_variants; ++i) {
       double t;
-      if ((st = time_launches(d, d->ops.row_step[i].fn, iters, &t)) != TTSH_OK) return st;
-      if (t < best) { best = t; br = i; btma = tma; }
+      if ((st = time_launches(d, d->ops.col_step[i].fn, iters, &t)) != TTSH_OK) return st;
+      if (t < best) { best = t; bc = i; }
     }
   }
-  d->dev.use_tma = btma;
-  best = 1e300;
-  for (int i = 0; i < d->ops.n_col_variants; ++i) {
-    double t;
-    if ((st = time_launches(d, d->ops.col_step[i].fn, iters, &t)) != TTSH_OK) return st;
-    if (t < best) { best = t; bc = i; }
-  }
-  d->dev.pdl = pdl0;
   d->dev.use_tma = tma0;
   if ((st = restore_state(d)) != TTSH_OK) return st;
   if ((st = ttsh_set_plan(d, br, bc)) != TTSH_OK) return st;

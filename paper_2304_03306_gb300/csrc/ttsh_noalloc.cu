@@ -153,8 +153,8 @@ extern "C" ttsh_status ttsh_step_noalloc(const ttsh_params* p, const void* K, vo
   // rebuild the row-pass inputs from the caller's state, then step
   e = ops.col(ttsh::K_COL_PROLOGUE, d, s);
   for (int64_t i = 0; i < nsteps && e == cudaSuccess; ++i) {
-    e = ops.row(ttsh::K_ROW_STEP, d, s);
-    if (e == cudaSuccess) e = ops.col(ttsh::K_COL_STEP, d, s);
+    e = ops.row_step[ops.alone_row].fn(d, s);
+    if (e == cudaSuccess) e = ops.col_step[ops.alone_col].fn(d, s);
   }
   if (e != cudaSuccess) return cuda_bad(e, "kernel launch");
   return TTSH_OK;

@@ -28,6 +28,7 @@ struct DomainDev {
   double cx, cy;   // centre for the order parameter
   int n;
   int pdl;         // launch the step kernels with programmatic dependent launch
+  int whole;       // never do (kernel timing: each launch runs by itself)
   int use_tma;     // let the row step kernel load its G tile with the TMA (where tma_ok)
   int* err;        // device status word (bounded waits that ran out)
   // G as a 2D tensor for the row pass's TMA loads, one map per row-block height R = 1, 2, 4
@@ -75,6 +76,7 @@ struct SizeOps {
   int n_row_variants, n_col_variants;           // entry 0 is the default tile shape
   StepVariant row_step[kMaxVariants];
   StepVariant col_step[kMaxVariants];
+  int alone_row, alone_col;   // fastest shapes of one domain stepped by itself (ttsh_step_noalloc)
   int args_bytes;                                    // size of one kernel argument block
   void (*pack_args)(const DomainDev&, void* dst);    // host copy of a domain's argument block
 };

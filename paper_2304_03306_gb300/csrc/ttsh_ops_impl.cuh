@@ -41,6 +41,15 @@ static int launch_smem(int smem, int grid, bool pdl) {
   return pdl && grid <= sm_count() && smem < kSpreadSmem ? kSpreadSmem : smem;
 }
 
+// Step kernels use programmatic dependent launch where the launch mode asks for it, and on grids
+// up to 512^2 in any case (results are the same bits): their passes take 3-6 us, of which the
+// overlap of one pass's start with the other's end saves 0.5 (256^2 float 8.47 -> 7.34 us a step,
+// 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1, in graphs; launched one by one the gap it
+// closes is larger: 256^2 12.0 us).  At 1024^2 it costs (22.7 -> 23.8 us), beyond it does nothing.
+constexpr int kPdlMaxN = 512;
+template <int N>
+static bool step_pdl(const DomainDev& d) { return !d.whole && (d.pdl || N <= kPdlMaxN); }
+
 // Launch, optionally as a programmatic dependent launch (the kernel may start while the
 // previous kernel in the stream is still running; it waits (griddepcontrol.wait) before it
 // touches anything that kernel writes) and optionally in clusters of `cl` blocks along x.
@@ -92,12 +101,14 @@ static cudaError_t launch_row_kind(const DomainDev& d, cudaStream_t s) {
       a.tma = 1;
     }
   }
-  const bool pdl = KIND == ROW_STEP && d.pdl;
+  const bool pdl = KIND == ROW_STEP && step_pdl<N>(d);
   return launch_k(row_kernel<T, N, KIND, R, PE, CL, CMP>, N / R, Geo::NT, launch_smem(Geo::SMEM, N / R, pdl), s, pdl,
                   CL, a, tm);
 }
 
-template <typename T, int N, int MODE, int PE = default_col_pe<T, N>()>
+// (the other column modes take the first step variant's shape, so that a state read back and set
+// again steps on bit for bit: the prologue makes the same row inputs as the step's column pass)
+template <typename T, int N, int MODE, int PE = default_step_col_pe<T, N>()>
 static cudaError_t launch_col_mode(const DomainDev& d, cudaStream_t s) {
   using Geo = ColGeo<T, N, MODE, PE>;
   static std::atomic<int> done{0};
@@ -105,7 +116,7 @@ static cudaError_t launch_col_mode(const DomainDev& d, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   // a recorded step adds one block that finishes the time-series sample
   const int extra = (MODE == COL_STEP && d.rec != nullptr) ? 1 : 0;
-  const bool pdl = MODE == COL_STEP && d.pdl;
+  const bool pdl = MODE == COL_STEP && step_pdl<N>(d);
   return launch_k(col_kernel<T, N, MODE, PE>, Geo::H + extra, Geo::NT, launch_smem(Geo::SMEM, Geo::H + extra, pdl), s,
                   pdl, 1, make_args<T>(d));
 }
@@ -218,6 +229,13 @@ static void add_col_variant(SizeOps& o) {
   }
 }
 
+// Index of the plain variant of this shape, 0 (the default) if there is none.
+inline int find_shape(const StepVariant* v, int n, int rows, int pe) {
+  for (int i = 0; i < n; ++i)
+    if (v[i].rows == rows && v[i].pe == pe && v[i].cl == 1 && v[i].cmp == 0) return i;
+  return 0;
+}
+
 template <typename T, int N>
 static SizeOps make_ops() {
   SizeOps o;
@@ -229,7 +247,8 @@ static SizeOps make_ops() {
   o.n_col_variants = 0;
   o.args_bytes = (int)sizeof(Args<T>);
   o.pack_args = &pack_args<T>;
-  add_row_variant<T, N, default_step_rows<T, N>(), default_step_row_pe<T, N>(), default_row_cluster<T, N>()>(o);
+  add_row_variant<T, N, default_step_rows<T, N>(), default_step_row_pe<T, N>(), default_row_cluster<T, N>(),
+                  default_step_compact<T, N>()>(o);
   add_col_variant<T, N, default_step_col_pe<T, N>()>(o);
   if constexpr (sizeof(T) == 4) {
     add_row_variant<T, N, 4, 16>(o);
@@ -257,6 +276,13 @@ static SizeOps make_ops() {
     add_col_variant<T, N, 8>(o);
     add_col_variant<T, N, 4>(o);
   }
+  // One domain by itself leaves most of the GPU idle up to 256^2: small tiles then spread it over
+  // more blocks and halve the butterflies of a thread's chain (float, us a step: 64^2 6.3 -> 4.9,
+  // 256^2 7.3 -> 6.0; double 64^2 26 -> 17, 256^2 40 -> 35).
+  constexpr bool F32 = sizeof(T) == 4;
+  o.alone_row = find_shape(o.row_step, o.n_row_variants, F32 ? (N <= 256 ? 2 : 4) : (N <= 256 ? 1 : 2),
+                           F32 ? (N <= 256 ? 8 : 16) : (N <= 256 ? 4 : 8));
+  o.alone_col = find_shape(o.col_step, o.n_col_variants, 1, F32 || N <= 256 ? 4 : 8);
   return o;
 }
 
