@@ -79,7 +79,7 @@ Layout layout_for(int n, size_t elt) {
   L.part = take(std::max((size_t)n * ttsh::kDiagQ * sizeof(double), (size_t)8192));
   L.colhist = take(H * (M + 1) * sizeof(double));
   L.bad = take(64);
-  L.out = take((8 + M + 1) * sizeof(double));
+  L.out = take((8 + M + 1 + 4) * sizeof(double));
   L.save = take(H * NK * 2 * elt + 64);   // state copy kept by ttsh_time_kernels
   L.rec = take((size_t)n * ttsh::kDiagQ * sizeof(double));   // time-series partials (<= n row blocks)
   L.recctl = take(64);                                        // time-series write position
@@ -407,13 +407,29 @@ __global__ void diag_reduce_kernel(const double* __restrict__ part, int nblocks,
   if (t < kDiagQ) out[t] = red[t][0];
 }
 
-__global__ void spectrum_reduce_kernel(const double* __restrict__ colhist, int ncols, int nbins,
-                                       double scale, double* __restrict__ out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nbins) return;
+// Shells' sums over the columns (only kx <= s + 1 reach shell s): 32 shells x 8 slices of the columns
+// a block, the slices added in order.  The last block also gathers the scalars a diagnostics call
+// returns behind the shells: mean flow, non-finite count, status word.
+template <typename T>
+__global__ void __launch_bounds__(256) spectrum_reduce_kernel(const double* __restrict__ colhist, int ncols, int nbins,
+                                                              double scale, const T* __restrict__ vmean,
+                                                              const int* __restrict__ bad, const int* __restrict__ err,
+                                                              double* __restrict__ out) {
+  __shared__ double red[8][32];
+  const int l = threadIdx.x & 31, sl = threadIdx.x >> 5, s = blockIdx.x * 32 + l;
+  const int top = s + 2 < ncols ? s + 2 : ncols;
   double acc = 0.0;
-  for (int c = 0; c < ncols; ++c) acc += colhist[(size_t)c * nbins + s];
-  out[s] = acc * scale;
+  if (s < nbins)
+    for (int c = sl; c < top; c += 8) acc += colhist[(size_t)c * nbins + s];
+  red[sl][l] = acc;
+  __syncthreads();
+  if (sl == 0 && s < nbins) {
+    double t = red[0][l];
+    for (int i = 1; i < 8; ++i) t += red[i][l];
+    out[s] = t * scale;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 4)
+    out[nbins + threadIdx.x] = threadIdx.x < 2 ? (double)vmean[threadIdx.x] : (double)(threadIdx.x == 2 ? *bad : *err);
 }
 
 void set_last_error(const char* msg) { g_last_error = msg; }
@@ -425,9 +441,10 @@ cudaError_t launch_diag_reduce(const double* part, int nblocks, double* out, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_spectrum_reduce(const double* colhist, int ncols, int nbins, double scale,
-                                   double* out, cudaStream_t s) {
-  spectrum_reduce_kernel<<<(nbins + 127) / 128, 128, 0, s>>>(colhist, ncols, nbins, scale, out);
+template <typename T>
+cudaError_t launch_spectrum_reduce(const DomainDev& d, int ncols, int nbins, double scale, cudaStream_t s) {
+  spectrum_reduce_kernel<T><<<(nbins + 31) / 32, 256, 0, s>>>(d.colhist, ncols, nbins, scale,
+                                                             static_cast<const T*>(d.vmean), d.bad, d.err, d.out + 8);
   return cudaGetLastError();
 }
 
@@ -1207,39 +1224,32 @@ ttsh_status ttsh_diagnostics(ttsh_domain* d, ttsh_diag* out, double* spectrum, i
   TTSH_CUDA(cudaMemsetAsync(d->dev.bad, 0, sizeof(int), s), "memset");
   TTSH_CUDA(d->ops.spec(d->dev, nb_dev, s), "spectrum kernel");
   const double scale = 1.0 / (2.0 * (double)d->n * (double)d->n);
-  TTSH_CUDA(ttsh::launch_spectrum_reduce(d->dev.colhist, d->H, nb_dev, scale, d->dev.out + 8, s), "spectrum reduce");
   // divergence of the real-space velocity: the diagnostic row pass left DFT_x[v_x], DFT_x[v_y]
   // in the inter-pass buffer; the column pass completes the transforms and takes the maxima
   TTSH_CUDA(cudaMemsetAsync(d->dev.out + 5, 0, 2 * sizeof(double), s), "memset");
   if ((st = run_col(d, ttsh::K_COL_DIV, s)) != TTSH_OK) return st;
-  std::vector<double> h(8 + nb_dev);
-  int bad = 0;
+  // last, so that everything the call returns is behind it in one piece
+  TTSH_CUDA(d->elt == sizeof(float) ? ttsh::launch_spectrum_reduce<float>(d->dev, d->H, nb_dev, scale, s)
+                                    : ttsh::launch_spectrum_reduce<double>(d->dev, d->H, nb_dev, scale, s),
+            "spectrum reduce");
+  std::vector<double> h(8 + nb_dev + 4);
   TTSH_CUDA(cudaMemcpyAsync(h.data(), d->dev.out, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s), "download diag");
-  TTSH_CUDA(cudaMemcpyAsync(&bad, d->dev.bad, sizeof(int), cudaMemcpyDeviceToHost, s), "download flag");
-  double vm[2];
-  if (d->elt == sizeof(float)) {
-    float f[2];
-    TTSH_CUDA(cudaMemcpyAsync(f, d->dev.vmean, sizeof(f), cudaMemcpyDeviceToHost, s), "download mean");
-    if ((st = sync(d, "diagnostics")) != TTSH_OK) return st;
-    vm[0] = f[0];
-    vm[1] = f[1];
-  } else {
-    TTSH_CUDA(cudaMemcpyAsync(vm, d->dev.vmean, sizeof(vm), cudaMemcpyDeviceToHost, s), "download mean");
-    if ((st = sync(d, "diagnostics")) != TTSH_OK) return st;
-  }
+  if ((st = sync(d, "diagnostics")) != TTSH_OK) return st;
+  const double *vm = h.data() + 8 + nb_dev, divmax = std::sqrt(h[5]), kvmax = std::sqrt(h[6]);
+  const int bad = (int)vm[2];
   const double inv2n2 = 1.0 / (2.0 * (double)d->n * (double)d->n);
   const double two_over_pi = 0.63661977236758134307553505349005744813783858296183;
   out->energy = h[0] * inv2n2;
   out->enstrophy = h[1] * inv2n2;
   out->psi = (h[2] / h[3] - two_over_pi) / (1.0 - two_over_pi);
-  out->max_div = h[6] > 0.0 ? h[5] / h[6] : 0.0;
+  out->max_div = kvmax > 0.0 ? divmax / kvmax : 0.0;
   out->mean_vx = vm[0] / d->n;
   out->mean_vy = vm[1] / d->n;
   out->step = d->steps;
   out->nonfinite = (int32_t)h[4] + bad;
   out->reserved = 0;
   for (int i = 0; i < nbins; ++i) spectrum[i] = i < nb_dev ? h[8 + i] : 0.0;
-  if ((st = check_status(d)) != TTSH_OK) return st;
+  if (vm[3] != 0.0 && (st = check_status(d)) != TTSH_OK) return st;
   if (out->nonfinite) return fail(TTSH_E_NONFINITE, "state holds non-finite values");
   return TTSH_OK;
 }

@@ -77,7 +77,7 @@ struct Args {
   double* rec;          // per-block time-series partials of a recorded step, or null
   RecCtl* recctl;       // with rec: where the column pass appends the step's sample
   int* err;             // device status word: 1 = a bounded wait in a kernel ran out
-  double* aux;          // two doubles: max |k.v^| and max |k||v^| of a divergence check
+  double* aux;          // two doubles: max |k.v^|^2 and max |k|^2 |v^|^2 of a divergence check
   int tma;              // 1: the row pass loads its G tile with the tensor-memory accelerator
   T a, b, lam, gv, gw, dt, dk, mean_decay;   // mean_decay = exp((a - 1) dt)
   double dx, cx, cy;    // grid spacing and the psi centre
@@ -686,21 +686,32 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
       A.K[(size_t)(y0 + r) * N + x] = k * k;          // K = (iDFT[...])^2
     }
   } else if constexpr (KIND == ROW_INV_DIAG) {
+    // Bound by the FP64 unit (a warp's double operation takes it 16 cycles): about 30 operations a
+    // point, with positions and squares of x shared by the block's rows, one reciprocal root
+    // instead of a root and a quotient, and the non-finite count kept as an integer (about 55 before).
+    // A diagnostics call of a 2048^2 float state, of which this pass took 438 us: 700 -> 454 us.
     double acc[kDiagQ] = {0, 0, 0, 0, 0};
-    for (int e = tid; e < R * N; e += NT) {
-      const int r = e / N, x = e % N;
-      const double w = (double)rl(0, r, x);
-      const double vx = (double)rl(1, r, x), vy = (double)rl(2, r, x);
+    int bad = 0;
+    double py[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) py[r] = (y0 + r - N / 2) * A.dx - A.cy;
+    for (int x = tid; x < N; x += NT) {
       const double px = (x - N / 2) * A.dx - A.cx;
-      const double py = (y0 + r - N / 2) * A.dx - A.cy;
-      const double rr = sqrt(px * px + py * py);
-      const double vn = sqrt(vx * vx + vy * vy);
-      acc[0] += vx * vx + vy * vy;
-      acc[1] += w * w;
-      acc[2] += rr > 0 ? fabs(-py * vx + px * vy) / rr : 0.0;
-      acc[3] += vn;
-      acc[4] += (isfinite(w) && isfinite(vx) && isfinite(vy)) ? 0.0 : 1.0;
+      const double px2 = px * px;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const T wt = rl(0, r, x), vxt = rl(1, r, x), vyt = rl(2, r, x);
+        const double w = (double)wt, vx = (double)vxt, vy = (double)vyt;
+        const double rr2 = fma(py[r], py[r], px2);
+        const double v2 = fma(vx, vx, vy * vy);
+        acc[0] += v2;
+        acc[1] = fma(w, w, acc[1]);
+        if (rr2 > 0) acc[2] = fma(fabs(fma(px, vy, -(py[r] * vx))), rsqrt(rr2), acc[2]);
+        acc[3] += sqrt(v2);
+        bad += (isfinite(wt) && isfinite(vxt) && isfinite(vyt)) ? 0 : 1;
+      }
     }
+    acc[4] = (double)bad;
     // fixed-order block reduction (deterministic)
     double* red = reinterpret_cast<double*>(smem_raw + Geo::OFF_RED);
     for (int q = 0; q < kDiagQ; ++q) red[q * 1024 + tid] = acc[q];
@@ -863,9 +874,11 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
     }
 
     if constexpr (MODE == COL_DIV) {
-      // largest |k.v^| and |k||v^| over the stored modes of the 1/2-rule disc, in double;
-      // maxima of non-negative doubles combine as their bit patterns (order-independent)
+      // largest |k.v^|^2 and |k|^2 |v^|^2 over the stored modes of the 1/2-rule disc, in double
+      // (the host takes the roots); maxima of non-negative doubles combine as their bit patterns
+      // (order-independent)
       double dmax = 0.0, kvmax = 0.0;
+      const double dk2 = (double)A.dk * (double)A.dk;
       for (int j = tid; j < NK; j += NT) {
         const int ky = ky_of(j);
         const int m2 = kx * kx + ky * ky;
@@ -1062,11 +1075,11 @@ __global__ void diag_reduce_kernel(const double* __restrict__ part, int nblocks,
 // Per-column shell spectrum: one thread per (stored column kx, shell s).  Shell s holds the
 // modes with round(|m|) = s, i.e. s^2 - s + 1 <= m^2 <= s^2 + s (s >= 1; s = 0: m = 0), so in
 // column kx its modes are two contiguous ranges of ky (ky >= 0 and ky < 0); each thread sums
-// them in the storage order of the column.  The s = 0 thread of each column also counts the
-// column's non-finite values.
+// them in the storage order of the column.  The first block of each column also counts the column's
+// non-finite values.
 __device__ __forceinline__ int isqrt_floor(long long v) {
   if (v <= 0) return 0;
-  long long r = (long long)sqrt((double)v);
+  long long r = (long long)sqrtf((float)v);   // within one of the root, corrected below
   while (r * r > v) --r;
   while ((r + 1) * (r + 1) <= v) ++r;
   return (int)r;
@@ -1078,8 +1091,13 @@ __global__ void spectrum_col_kernel(Args<T> A, int nbins, double* __restrict__ c
   constexpr int M = N / 4, NK = 2 * M + 1;
   const int kx = blockIdx.y;
   const int sh = blockIdx.x * blockDim.x + threadIdx.x;
-  if (sh >= nbins) return;
   const cplx<T>* col = A.what + (size_t)kx * NK;
+  if (blockIdx.x == 0) {
+    int bad = 0;
+    for (int j = threadIdx.x; j < NK; j += blockDim.x) bad += isfinite(col[j].x) && isfinite(col[j].y) ? 0 : 1;
+    if (bad) atomicAdd(badcount, bad);
+  }
+  if (sh >= nbins) return;
   const double dk = (double)A.dk;
   const double wgt = kx > 0 ? 2.0 : 1.0;   // mx > 0 columns stand for +-mx
   auto energy = [&](int ky) {
@@ -1105,15 +1123,11 @@ __global__ void spectrum_col_kernel(Args<T> A, int nbins, double* __restrict__ c
     for (int ky = -top; ky <= -nlo; ++ky) h += wgt * energy(ky);
   }
   colhist[(size_t)kx * nbins + sh] = h;
-  if (sh == 0) {
-    int bad = 0;
-    for (int j = 0; j < NK; ++j)
-      if (!isfinite((double)col[j].x) || !isfinite((double)col[j].y)) ++bad;
-    if (bad) atomicAdd(badcount, bad);
-  }
 }
 
-__global__ void spectrum_reduce_kernel(const double* __restrict__ colhist, int ncols, int nbins,
-                                       double scale, double* __restrict__ out);
+template <typename T>
+__global__ void spectrum_reduce_kernel(const double* __restrict__ colhist, int ncols, int nbins, double scale,
+                                       const T* __restrict__ vmean, const int* __restrict__ bad,
+                                       const int* __restrict__ err, double* __restrict__ out);
 
 }  // namespace ttsh

@@ -20,7 +20,8 @@ struct DomainDev {
   double* part;    // row-block diagnostic partials
   double* colhist; // H x (N/4 + 1) spectrum partials
   int* bad;        // non-finite counter
-  double* out;     // reduced diagnostics (8 doubles: 5 sums, 2 divergence maxima, 1 spare) + spectrum bins
+  double* out;     // reduced diagnostics (8 doubles: 5 sums, 2 divergence maxima, 1 spare), spectrum
+                   // bins, then mean flow (2), non-finite count, status word
   unsigned char* knaive;   // binary mask K_naive as given (1 = masked), N x N bytes
   double* rec;     // time-series partials of a recorded step (null: plain step)
   void* recctl;    // time-series write position (RecCtl), used with rec
@@ -134,7 +135,5 @@ int domain_refresh_on(ttsh_domain* d, cudaStream_t s);   // on another stream (g
 int domain_clone(const ttsh_domain* src, ttsh_domain** out);
 
 cudaError_t launch_diag_reduce(const double* part, int nblocks, double* out, cudaStream_t s);
-cudaError_t launch_spectrum_reduce(const double* colhist, int ncols, int nbins, double scale,
-                                   double* out, cudaStream_t s);
 
 }  // namespace ttsh
