@@ -160,7 +160,7 @@ __host__ __device__ constexpr int smem_blocks_per_sm(int smem) { return (228 * 1
 // forward transforms work in place (no separate buffers) and the mask rows are read from
 // global memory where the real-space terms need them (not staged), so that two or more
 // blocks fit per SM on large grids and one block's staging and stores overlap another's
-// transforms.
+// transforms.  CMP = 2: in place, the mask rows staged.
 template <typename T, int N, int KIND, int R, int PEV, int CL = 1, int CMP = 0>
 struct RowGeo {
   static constexpr int L = N / 2, M = N / 4, H = M + 1;
@@ -186,7 +186,7 @@ struct RowGeo {
   static constexpr int GIN_DENSE = NPL * align128(HC * RS * CB);   // decides what is staged
   static constexpr int KS_BYTES = KIND == ROW_STEP ? align16(R * N * (int)sizeof(T)) : 0;
   static constexpr int RED_BYTES = KIND == ROW_INV_DIAG ? kDiagQ * 1024 * 8 : 0;
-  static constexpr bool STAGE_K = KS_BYTES > 0 && CMP == 0 && TW_BYTES + BUF_BYTES + KS_BYTES + RED_BYTES <= kSmemLimit;
+  static constexpr bool STAGE_K = KS_BYTES > 0 && CMP != 1 && TW_BYTES + BUF_BYTES + KS_BYTES + RED_BYTES <= kSmemLimit;
   static constexpr bool STAGE_G = GIN_DENSE > 0 &&
       TW_BYTES + BUF_BYTES + GIN_DENSE + (STAGE_K ? KS_BYTES : 0) + RED_BYTES <= kSmemLimit;
   // step kernel: the forward transforms get buffers of their own when they fit, so that the
@@ -240,7 +240,9 @@ struct RowGeo {
 };
 
 // Column-pass geometry and shared-memory plan.
-template <typename T, int N, int MODE, int PEV>
+// LEAN = 1: the forward inputs are staged straight into the transform buffers, without an area of
+// their own (less shared memory, one barrier more; the same values).
+template <typename T, int N, int MODE, int PEV, int LEAN = 0>
 struct ColGeo {
   static constexpr int M = N / 4, H = M + 1, NK = 2 * M + 1;
   static constexpr int PE = cmin(PEV, N);
@@ -262,7 +264,7 @@ struct ColGeo {
   // forward inputs in one batch: the NF columns can come as bulk copies (contiguous in Rr)
   // into an unpadded staging area that the first transform stage reads
   static constexpr int STG_BYTES = NF * N * CB;
-  static constexpr bool BULK = NF > 0 && FB >= NF && FIXED + FB * LP * CB + STG_BYTES <= kSmemLimit;
+  static constexpr bool BULK = LEAN == 0 && NF > 0 && FB >= NF && FIXED + FB * LP * CB + STG_BYTES <= kSmemLimit;
   static constexpr int OFF_BUF = TW_BYTES;
   static constexpr int OFF_ACC = OFF_BUF + align16(FB * LP * CB);
   static constexpr int OFF_WS = OFF_ACC + ACC_BYTES;
@@ -775,9 +777,9 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
 // ---------------------------------------------------------------------------------------
 // Column pass body (one block = stored column mx = kx)
 // ---------------------------------------------------------------------------------------
-template <typename T, int N, int MODE, int PEV>
+template <typename T, int N, int MODE, int PEV, int LEAN = 0>
 __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char* smem_raw) {
-  using Geo = ColGeo<T, N, MODE, PEV>;
+  using Geo = ColGeo<T, N, MODE, PEV, LEAN>;
   static_assert(Geo::VALID, "column pass tile does not fit");
   constexpr int M = Geo::M, H = Geo::H, NK = Geo::NK;
   constexpr int PE = Geo::PE, PS = Geo::PS, LP = Geo::LP, NT = Geo::NT, FB = Geo::FB;
@@ -884,9 +886,8 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
         const int m2 = kx * kx + ky * ky;
         if (m2 > M * M) continue;
         const double ax = (double)acc[j].x, ay = (double)acc[j].y;
-        const double dkd = (double)A.dk;
-        dmax = fmax(dmax, sqrt(ax * ax + ay * ay));
-        kvmax = fmax(kvmax, dkd * sqrt((double)m2) * sqrt((double)ws[j].x));
+        dmax = fmax(dmax, fma(ax, ax, ay * ay));
+        kvmax = fmax(kvmax, dk2 * (double)m2 * (double)ws[j].x);
       }
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {

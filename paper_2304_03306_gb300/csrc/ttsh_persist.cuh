@@ -98,13 +98,23 @@ __device__ __forceinline__ bool wait_count(const unsigned long long* ctr, unsign
 // Sizes the persistent kernel holds (the batched sweeps' grids and smaller).
 constexpr int kPersistMaxN = 512;
 
+// Float bodies in the forms with the least shared memory (the same values as the per-launch ones,
+// see CMP and LEAN): the stepper is bound by how many items an SM holds at once (30 KB a block
+// instead of 44).  48-domain sweep, 160 steps with the states read: 11.8 ms with the per-launch
+// forms at 5 blocks an SM; in place at 5 blocks 10.9, at 6 10.6, at 7 10.5 (spilling); with the
+// mask rows read from global memory as well 10.8.
+constexpr int kPersistCmp = 2;
+constexpr int kPersistBlocks = 6;   // resident blocks per SM the float kernel is compiled for
+
 template <typename T, int N>
 struct PersistShape {
   static constexpr int R = default_step_rows<T, N>();
   static constexpr int RPE = default_step_row_pe<T, N>();
   static constexpr int CPE = default_step_col_pe<T, N>();
-  using RG = RowGeo<T, N, ROW_STEP, R, RPE>;
-  using CG = ColGeo<T, N, COL_STEP, CPE>;
+  static constexpr int CMP = sizeof(T) == 4 ? kPersistCmp : 0;
+  static constexpr int LEAN = sizeof(T) == 4 ? 1 : 0;
+  using RG = RowGeo<T, N, ROW_STEP, R, RPE, 1, CMP>;
+  using CG = ColGeo<T, N, COL_STEP, CPE, LEAN>;
   static constexpr int NT = cmax(RG::NT, CG::NT);
   static constexpr int SMEM = cmax(RG::SMEM, CG::SMEM);
 };
@@ -129,7 +139,7 @@ __device__ __noinline__ void persist_row(const Args<T>& Ag, int blk, unsigned ch
   using S = PersistShape<T, N>;
   if (threadIdx.x < S::RG::NT) {
     const Args<T> A = Ag;
-    row_body<T, N, ROW_STEP, S::R, S::RPE, 1, 0, false>(A, blk, smem, nullptr);
+    row_body<T, N, ROW_STEP, S::R, S::RPE, 1, S::CMP, false>(A, blk, smem, nullptr);
   }
 }
 template <typename T, int N>
@@ -137,7 +147,7 @@ __device__ __noinline__ void persist_col(const Args<T>& Ag, int blk, unsigned ch
   using S = PersistShape<T, N>;
   if (threadIdx.x < S::CG::NT) {
     const Args<T> A = Ag;
-    col_body<T, N, COL_STEP, S::CPE>(A, blk, smem);
+    col_body<T, N, COL_STEP, S::CPE, S::LEAN>(A, blk, smem);
   }
 }
 template <typename T, int N>
@@ -168,7 +178,7 @@ __device__ __forceinline__ void item_need(const PDomain<T>* doms, const PItem& i
 // Published items alternate between two slots, so a slot is never rewritten while a thread
 // may still read it.
 template <typename T>
-__global__ void __launch_bounds__(PersistLimits<T>::NT + 32, sizeof(T) == 4 ? 5 : 2)
+__global__ void __launch_bounds__(PersistLimits<T>::NT + 32, sizeof(T) == 4 ? kPersistBlocks : 2)
 persistent_step_kernel(const PDomain<T>* __restrict__ doms, const PItem* __restrict__ items, int ips,
                        long long nsteps, unsigned long long* __restrict__ ctl, unsigned long long limit_ns) {
   constexpr int NB = PersistLimits<T>::NT;
