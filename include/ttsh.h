@@ -206,7 +206,8 @@ ttsh_status ttsh_time_kernels(ttsh_domain* d, int32_t iters, double* ms);
 
 /* Step-kernel tile shapes ("plan").  Each grid size has a list of row-pass variants (rows
  * per block, points per thread of the register butterflies) and column-pass variants
- * (points per thread); entry 0 is the default.  Variants compute the same step with a
+ * (points per thread); a domain starts with the entry measured
+ * fastest for its size (entry 0 where batches take that size).  Variants compute the same step with a
  * different factorisation of the transforms, so results agree to rounding, not bit for bit.
  * ttsh_autotune times every variant (as ttsh_time_kernels does, `iters` launches each, state
  * restored) and selects the fastest row and column variant.  plan (10 int32, may be NULL):

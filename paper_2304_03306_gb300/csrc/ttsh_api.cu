@@ -891,7 +891,7 @@ ttsh_status ttsh_create_domain(const uint8_t* mask, const ttsh_params* p, void* 
   d->steps = 0;
   d->graph = nullptr;
   d->graph_len = 0;
-  d->rv = 0;
+  d->rv = ops.start_row;
   d->cv = 0;
   d->lay = layout_for(d->n, d->elt);
   d->owns_ws = workspace == nullptr;

@@ -121,9 +121,8 @@ __host__ __device__ constexpr int default_col_pe() { return sizeof(T) == 4 ? (N 
 // 3.7 us per row pass - but slower in a batch, where twice the blocks pay their fixed costs
 // twice: 53.0 against 49.9 us per step of the 48-domain sweep; so they stay autotuner
 // choices.)
-// The larger grids start with the shapes measured fastest: 2048^2 the compact two-row pass (50.8
-// us; the plain one 58.1), 4096^2 two rows (238 us; one row 327), 1024^2 a 16-point column pass
-// (7.8 us; 8-point 8.1).  Double up to 256^2: one row and 4 points per thread in both passes
+// The larger grids start with the shapes measured fastest: 4096^2 two rows (238 us; one row 327),
+// 1024^2 a 16-point column pass (7.8 us; 8-point 8.1).  Double up to 256^2: one row and 4 points per thread in both passes
 // (64^2 27 -> 17 us a step, 256^2 41 -> 35), in batches as well.
 template <typename T, int N>
 __host__ __device__ constexpr int default_step_rows() {
@@ -137,8 +136,6 @@ template <typename T, int N>
 __host__ __device__ constexpr int default_step_col_pe() {
   return sizeof(T) == 4 ? (N == 512 || N == 1024 ? 16 : default_col_pe<T, N>()) : (N <= 256 ? 4 : default_col_pe<T, N>());
 }
-template <typename T, int N>
-__host__ __device__ constexpr int default_step_compact() { return sizeof(T) == 4 && N == 2048 ? 1 : 0; }
 // blocks per cluster of the default step row pass (8192^2 float: one row per block, pairs)
 template <typename T, int N>
 __host__ __device__ constexpr int default_row_cluster() { return sizeof(T) == 4 && N >= 8192 ? 2 : 1; }
