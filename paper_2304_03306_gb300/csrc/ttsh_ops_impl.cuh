@@ -41,14 +41,15 @@ static int launch_smem(int smem, int grid, bool pdl) {
   return pdl && grid <= sm_count() && smem < kSpreadSmem ? kSpreadSmem : smem;
 }
 
-// Step kernels use programmatic dependent launch where the launch mode asks for it, and on grids
-// up to 512^2 in any case (results are the same bits): their passes take 3-6 us, of which the
-// overlap of one pass's start with the other's end saves 0.5 (256^2 float 8.47 -> 7.34 us a step,
-// 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1, in graphs; launched one by one the gap it
-// closes is larger: 256^2 12.0 us).  At 1024^2 it costs (22.7 -> 23.8 us), beyond it does nothing.
+// Step kernels use programmatic dependent launch where the launch mode asks for it, when they
+// are launched one by one, and in graphs on grids up to 512^2 (results are the same bits).  One
+// by one the overlap hides the gap between launches (us a step: 256^2 float 12.0 -> 7.8, 1024^2
+// 26.8 -> 23.4, 2048^2 87.2 -> 81.9); in a graph it saves 0.5 us of a small grid's pass (256^2
+// 8.47 -> 7.34 us a step, 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1) but costs at 1024^2
+// (22.7 -> 23.8) and does nothing beyond.
 constexpr int kPdlMaxN = 512;
 template <int N>
-static bool step_pdl(const DomainDev& d) { return !d.whole && (d.pdl || N <= kPdlMaxN); }
+static bool step_pdl(const DomainDev& d) { return !d.whole && (d.pdl || !d.captured || N <= kPdlMaxN); }
 
 // Launch, optionally as a programmatic dependent launch (the kernel may start while the
 // previous kernel in the stream is still running; it waits (griddepcontrol.wait) before it
