@@ -513,8 +513,17 @@ int domain_n(const ttsh_domain* d) { return d->n; }
 double domain_dx(const ttsh_domain* d) { return d->p.dx; }
 int domain_fields_to_staging(ttsh_domain* d) { return run_row(d, K_ROW_INV_FIELDS, d->stream); }
 void domain_add_steps(ttsh_domain* d, int64_t n) { d->steps += n; }
-int domain_add_vorticity_from_staging(ttsh_domain* d) {
-  ttsh_status st = run_row(d, K_ROW_FWD_MASK, d->stream);   // one real field forward
+int domain_features(ttsh_domain* d, float* feat, const float* fscale) {
+  FieldIo& io = d->dev.io;
+  io.feat = feat;
+  for (int i = 0; i < 4; ++i) io.fscale[i] = fscale[i];
+  io.feat16 = reinterpret_cast<uintptr_t>(feat) % 16 == 0;
+  return run_row(d, K_ROW_FEATURES, d->stream);
+}
+int domain_add_vorticity(ttsh_domain* d, const float* field, float scale) {
+  d->dev.io.corr = field;
+  d->dev.io.cscale = scale;
+  ttsh_status st = run_row(d, K_ROW_FWD_CORR, d->stream);
   if (st != TTSH_OK) return st;
   return run_col(d, K_COL_ADDW, d->stream);
 }

@@ -818,28 +818,10 @@ __global__ void pointwise_weights_kernel(const float* __restrict__ W, __nv_bfloa
   Wn[e] = __float2bfloat16_rn(W[e]);
 }
 
-// Input channels of sample b from a domain's staging (omega, v_x, v_y as doubles) and K
-template <typename T>
-__global__ void features_kernel(const double* __restrict__ real, const T* __restrict__ K, long long nn,
-                                float s0, float s1, float s2, float s3, float* __restrict__ x) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nn) return;
-  x[p * 4 + 0] = (float)real[p] * s0;
-  x[p * 4 + 1] = (float)real[nn + p] * s1;
-  x[p * 4 + 2] = (float)real[2 * nn + p] * s2;
-  x[p * 4 + 3] = (float)K[p] * s3;
-}
-
 __global__ void diff_kernel(const double* __restrict__ a, const double* __restrict__ b, long long n, float scale,
                             float* __restrict__ out) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) out[p] = (float)(a[p] - b[p]) * scale;
-}
-
-__global__ void to_double_scaled_kernel(const float* __restrict__ src, long long n, float scale,
-                                        double* __restrict__ dst) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n) dst[p] = (double)src[p] * (double)scale;
 }
 
 // Adam with bias correction on the FP32 master weights and the BF16 copies of the mixing weights in the same pass: parameter i
@@ -1749,20 +1731,7 @@ ttsh_status ttsh_fno_features(ttsh_fno* f, ttsh_domain* d, float* x, int32_t sam
   if (!f || !d || !x) return fno_fail(TTSH_E_INVALID, "NULL argument");
   if (ttsh::domain_n(d) != f->n) return fno_fail(TTSH_E_INVALID, "domain grid differs from the network's");
   if (sample < 0 || sample >= f->Bmax) return fno_fail(TTSH_E_INVALID, "sample out of range");
-  ttsh_status st = (ttsh_status)ttsh::domain_fields_to_staging(d);
-  if (st != TTSH_OK) return st;
-  cudaStream_t s = ttsh::domain_stream(d);
-  const ttsh::DomainDev* dv = ttsh::domain_dev(d);
-  float* xs = x + (long long)sample * f->nn * 4;
-  const unsigned blk = (unsigned)((f->nn + 255) / 256);
-  if (ttsh::domain_precision(d) == 32)
-    features_kernel<float><<<blk, 256, 0, s>>>(dv->real, (const float*)dv->K, f->nn, f->in_scale[0], f->in_scale[1],
-                                                f->in_scale[2], f->in_scale[3], xs);
-  else
-    features_kernel<double><<<blk, 256, 0, s>>>(dv->real, (const double*)dv->K, f->nn, f->in_scale[0],
-                                                 f->in_scale[1], f->in_scale[2], f->in_scale[3], xs);
-  FNO_CUDA(cudaGetLastError(), "features");
-  return TTSH_OK;
+  return (ttsh_status)ttsh::domain_features(d, x + (long long)sample * f->nn * 4, f->in_scale);
 }
 
 ttsh_status ttsh_fno_rollout(ttsh_fno* f, ttsh_domain* d, int64_t nsteps, int32_t correct_every, float* scratch) {
@@ -1844,11 +1813,7 @@ ttsh_status ttsh_fno_correct(ttsh_fno* f, ttsh_domain* d, float* scratch) {
   st = forward_impl(f, scratch, 1, y, nullptr, nullptr);
   f->stream = keep;
   if (st != TTSH_OK) return st;
-  const ttsh::DomainDev* dv = ttsh::domain_dev(d);
-  to_double_scaled_kernel<<<(unsigned)((f->nn + 255) / 256), 256, 0, ttsh::domain_stream(d)>>>(
-      y, f->nn, 1.f / f->out_scale, dv->real);
-  FNO_CUDA(cudaGetLastError(), "correction");
-  return (ttsh_status)ttsh::domain_add_vorticity_from_staging(d);
+  return (ttsh_status)ttsh::domain_add_vorticity(d, y, 1.f / f->out_scale);
 }
 
 }  // extern "C"

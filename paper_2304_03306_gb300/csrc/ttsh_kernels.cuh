@@ -43,6 +43,7 @@
 #include <cuda.h>   // CUtensorMap (the tensor-map descriptor of the TMA loads)
 
 #include "ttsh_fft.cuh"
+#include "ttsh_ops.h"
 #include "ttsh_wait.cuh"
 
 namespace ttsh {
@@ -84,7 +85,7 @@ struct Args {
 };
 
 enum RowKind { ROW_STEP = 0, ROW_FWD_VEL = 1, ROW_FWD_MASK = 2, ROW_INV_FIELDS = 3,
-               ROW_INV_MASK = 4, ROW_INV_DIAG = 5 };
+               ROW_INV_MASK = 4, ROW_INV_DIAG = 5, ROW_FEATURES = 6, ROW_FWD_CORR = 7 };
 enum ColMode { COL_STEP = 0, COL_PROLOGUE = 1, COL_PROJECT = 2, COL_MASK = 3, COL_ADDW = 4, COL_DIV = 5 };
 
 constexpr int kDiagQ = 5;   // per-block partials: sum|v|^2, sum w^2, sum|e_th.v|, sum|v|, #nonfinite
@@ -95,12 +96,12 @@ __host__ __device__ constexpr int align16(int v) { return (v + 15) / 16 * 16; }
 __host__ __device__ constexpr int align128(int v) { return (v + 127) / 128 * 128; }
 
 template <int KIND> __host__ __device__ constexpr int row_inv_fields() {
-  return KIND == ROW_STEP ? 3 : KIND == ROW_INV_FIELDS ? 3 : KIND == ROW_INV_DIAG ? 3
+  return KIND == ROW_STEP ? 3 : KIND == ROW_INV_FIELDS || KIND == ROW_FEATURES ? 3 : KIND == ROW_INV_DIAG ? 3
        : KIND == ROW_INV_MASK ? 1 : 0;
 }
 // (the diagnostic pass also forward-transforms v_x, v_y for the divergence check)
 template <int KIND> __host__ __device__ constexpr int row_fwd_fields() {
-  return KIND == ROW_STEP ? 3 : KIND == ROW_FWD_VEL ? 2 : KIND == ROW_FWD_MASK ? 1 : KIND == ROW_INV_DIAG ? 2 : 0;
+  return KIND == ROW_STEP ? 3 : KIND == ROW_FWD_VEL ? 2 : KIND == ROW_FWD_MASK || KIND == ROW_FWD_CORR ? 1 : KIND == ROW_INV_DIAG ? 2 : 0;
 }
 
 // Default tile shapes (the autotuner may pick others for the step kernels).
@@ -485,7 +486,7 @@ __device__ __forceinline__ void dsmem_st(unsigned a, cplx<double> v) {
 // REC = false leaves out the time-series sums (for callers whose Args never carry them).
 template <typename T, int N, int KIND, int R, int PEV, int CL = 1, int CMP = 0, bool REC = true>
 __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned char* smem_raw,
-                                         const CUtensorMap* tmapG) {
+                                         const CUtensorMap* tmapG, const FieldIo* io = nullptr) {
   using Geo = RowGeo<T, N, KIND, R, PEV, CL, CMP>;
   static_assert(Geo::VALID, "row pass tile does not fit");
   constexpr int L = Geo::L, M = Geo::M, H = Geo::H;
@@ -677,6 +678,27 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
       const int t = e / N;
       const int r = t % R, f = t / R;
       A.real[((size_t)f * N + (y0 + r)) * N + x] = (double)rl(f, r, x);
+    }
+  } else if constexpr (KIND == ROW_FEATURES) {
+    for (int e = tid; e < R * N; e += NT) {
+      const int r = e / N, x = e % N;
+      const size_t p = (size_t)(y0 + r) * N + x;
+      const float4 f = make_float4((float)rl(0, r, x) * io->fscale[0], (float)rl(1, r, x) * io->fscale[1],
+                                   (float)rl(2, r, x) * io->fscale[2], (float)A.K[p] * io->fscale[3]);
+      float* o = io->feat + 4 * p;
+      if (io->feat16) {
+        *reinterpret_cast<float4*>(o) = f;
+      } else {
+        o[0] = f.x;
+        o[1] = f.y;
+        o[2] = f.z;
+        o[3] = f.w;
+      }
+    }
+  } else if constexpr (KIND == ROW_FWD_CORR) {
+    for (int e = tid; e < R * N; e += NT) {
+      const int r = e / N, x = e % N;
+      rl(0, r, x) = (T)((double)io->corr[(size_t)(y0 + r) * N + x] * (double)io->cscale);
     }
   } else if constexpr (KIND == ROW_INV_MASK) {
     for (int e = tid; e < R * N; e += NT) {
@@ -1031,6 +1053,14 @@ __global__ void __launch_bounds__(RowGeo<T, N, KIND, R, PEV, CL, CMP>::NT)
 row_kernel(Args<T> A, const __grid_constant__ CUtensorMap tmapG) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   row_body<T, N, KIND, R, PEV, CL, CMP>(A, blockIdx.x, smem_base128(smem_raw), &tmapG);
+}
+
+// Row kinds that exchange fields with the corrector network.
+template <typename T, int N, int KIND, int R, int PEV>
+__global__ void __launch_bounds__(RowGeo<T, N, KIND, R, PEV>::NT)
+row_io_kernel(Args<T> A, FieldIo io) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  row_body<T, N, KIND, R, PEV>(A, blockIdx.x, smem_base128(smem_raw), nullptr, &io);
 }
 
 template <typename T, int N, int MODE, int PEV>

@@ -8,6 +8,15 @@
 
 namespace ttsh {
 
+// Real fields exchanged with the corrector network, in its FP32 (K_ROW_FEATURES, K_ROW_FWD_CORR).
+struct FieldIo {
+  float* feat;        // [N][N][4]: (omega, v_x, v_y, K) times fscale
+  const float* corr;  // [N][N]: a vorticity correction, times cscale
+  float fscale[4];
+  float cscale;
+  int feat16;         // 1: feat is 16-byte aligned
+};
+
 // Device pointers and constants of one domain, independent of the arithmetic type.
 struct DomainDev {
   void* what;      // omega^ half-spectrum, H x NK complex
@@ -37,10 +46,11 @@ struct DomainDev {
   // (tma_ok[i] = 0 where the shape does not allow it or the map could not be made)
   CUtensorMap tmapG[3];
   int tma_ok[3];
+  FieldIo io;      // set by the caller of the two row kinds that use it
 };
 
 enum { K_ROW_STEP = 0, K_ROW_FWD_VEL = 1, K_ROW_FWD_MASK = 2, K_ROW_INV_FIELDS = 3,
-       K_ROW_INV_MASK = 4, K_ROW_INV_DIAG = 5 };
+       K_ROW_INV_MASK = 4, K_ROW_INV_DIAG = 5, K_ROW_FEATURES = 6, K_ROW_FWD_CORR = 7 };
 enum { K_COL_STEP = 0, K_COL_PROLOGUE = 1, K_COL_PROJECT = 2, K_COL_MASK = 3, K_COL_ADDW = 4, K_COL_DIV = 5 };
 
 using RowFn = cudaError_t (*)(int kind, const DomainDev&, cudaStream_t);
@@ -124,9 +134,11 @@ int domain_n(const ttsh_domain* d);
 double domain_dx(const ttsh_domain* d);
 // Real-space omega, v_x, v_y of the state into the domain's double staging planes 0..2.
 int domain_fields_to_staging(ttsh_domain* d);
-// Add the real field in staging plane 0 to omega (projected onto the 1/2-rule disc,
-// Hermitian, zero mean) and refresh the inter-pass buffers.
-int domain_add_vorticity_from_staging(ttsh_domain* d);
+// (omega, v_x, v_y, K) of the state, scaled, as the network's FP32 input.
+int domain_features(ttsh_domain* d, float* feat, const float* fscale);
+// Add a real field times `scale` to omega (projected onto the 1/2-rule disc, Hermitian, zero
+// mean) and refresh the inter-pass buffers.
+int domain_add_vorticity(ttsh_domain* d, const float* field, float scale);
 // Adjust the step counter (for steps replayed from a graph the domain did not record).
 void domain_add_steps(ttsh_domain* d, int64_t n);
 double domain_dt(const ttsh_domain* d);

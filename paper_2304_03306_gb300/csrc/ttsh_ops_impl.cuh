@@ -122,6 +122,17 @@ static cudaError_t launch_col_mode(const DomainDev& d, cudaStream_t s) {
                   pdl, 1, make_args<T>(d));
 }
 
+template <typename T, int N, int KIND>
+static cudaError_t launch_row_io(const DomainDev& d, cudaStream_t s) {
+  constexpr int R = default_rows<T, N>(), PE = default_row_pe<T, N>();
+  using Geo = RowGeo<T, N, KIND, R, PE>;
+  static std::atomic<int> done{0};
+  cudaError_t e = set_smem(row_io_kernel<T, N, KIND, R, PE>, Geo::SMEM, done);
+  if (e != cudaSuccess) return e;
+  row_io_kernel<T, N, KIND, R, PE><<<N / R, Geo::NT, Geo::SMEM, s>>>(make_args<T>(d), d.io);
+  return cudaGetLastError();
+}
+
 template <typename T, int N>
 static cudaError_t launch_row(int kind, const DomainDev& d, cudaStream_t s) {
   switch (kind) {
@@ -131,6 +142,8 @@ static cudaError_t launch_row(int kind, const DomainDev& d, cudaStream_t s) {
     case K_ROW_INV_FIELDS: return launch_row_kind<T, N, ROW_INV_FIELDS>(d, s);
     case K_ROW_INV_MASK: return launch_row_kind<T, N, ROW_INV_MASK>(d, s);
     case K_ROW_INV_DIAG: return launch_row_kind<T, N, ROW_INV_DIAG>(d, s);
+    case K_ROW_FEATURES: return launch_row_io<T, N, ROW_FEATURES>(d, s);
+    case K_ROW_FWD_CORR: return launch_row_io<T, N, ROW_FWD_CORR>(d, s);
   }
   return cudaErrorInvalidValue;
 }
