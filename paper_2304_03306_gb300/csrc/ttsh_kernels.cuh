@@ -1100,11 +1100,10 @@ col_kernel_batched(const Args<T>* __restrict__ args) {
 // Sum nblocks x kDiagQ partials into out[kDiagQ] with one block of 256 threads.
 __global__ void diag_reduce_kernel(const double* __restrict__ part, int nblocks, double* out);
 
-// Per-column shell spectrum: one thread per (stored column kx, shell s).  Shell s holds the
+// Per-column shell spectrum: a block per stored column kx, a thread per shell s.  Shell s holds the
 // modes with round(|m|) = s, i.e. s^2 - s + 1 <= m^2 <= s^2 + s (s >= 1; s = 0: m = 0), so in
 // column kx its modes are two contiguous ranges of ky (ky >= 0 and ky < 0); each thread sums
-// them in the storage order of the column.  The first block of each column also counts the column's
-// non-finite values.
+// them in the storage order of the column.  The block also counts the column's non-finite values.
 __device__ __forceinline__ int isqrt_floor(long long v) {
   if (v <= 0) return 0;
   long long r = (long long)sqrtf((float)v);   // within one of the root, corrected below
@@ -1114,43 +1113,45 @@ __device__ __forceinline__ int isqrt_floor(long long v) {
 }
 
 template <typename T, int N>
-__global__ void spectrum_col_kernel(Args<T> A, int nbins, double* __restrict__ colhist,
-                                    int* __restrict__ badcount) {
+__global__ void __launch_bounds__(256) spectrum_col_kernel(Args<T> A, int nbins, double* __restrict__ colhist,
+                                                           int* __restrict__ badcount) {
   constexpr int M = N / 4, NK = 2 * M + 1;
-  const int kx = blockIdx.y;
-  const int sh = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double en[NK];   // energy of each mode of the column (one quotient a mode, in parallel)
+  const int kx = blockIdx.x;
   const cplx<T>* col = A.what + (size_t)kx * NK;
-  if (blockIdx.x == 0) {
-    int bad = 0;
-    for (int j = threadIdx.x; j < NK; j += blockDim.x) bad += isfinite(col[j].x) && isfinite(col[j].y) ? 0 : 1;
-    if (bad) atomicAdd(badcount, bad);
-  }
-  if (sh >= nbins) return;
   const double dk = (double)A.dk;
   const double wgt = kx > 0 ? 2.0 : 1.0;   // mx > 0 columns stand for +-mx
-  auto energy = [&](int ky) {
+  int bad = 0;
+  for (int j = threadIdx.x; j < NK; j += 256) {
+    const cplx<T> w = col[j];
+    const int ky = j <= M ? j : j - NK;
     const int m2 = kx * kx + ky * ky;
     if (m2 == 0) {
       const double u = (double)A.vmean[0], v = (double)A.vmean[1];
-      return u * u + v * v;
+      en[j] = u * u + v * v;
+    } else {
+      const double wr = (double)w.x, wi = (double)w.y;
+      en[j] = (wr * wr + wi * wi) / (dk * dk * (double)m2);
     }
-    const cplx<T> w = col[ky >= 0 ? ky : ky + NK];
-    const double wr = (double)w.x, wi = (double)w.y;
-    return (wr * wr + wi * wi) / (dk * dk * (double)m2);
-  };
-  double h = 0.0;
-  const long long s2 = (long long)sh * sh;
-  const long long lo2 = sh == 0 ? 0 : s2 - sh + 1, hi2 = sh == 0 ? 0 : s2 + sh;   // range of m^2
-  const long long k2 = (long long)kx * kx;
-  if (hi2 >= k2) {
-    const int ylo = lo2 - k2 <= 0 ? 0 : isqrt_floor(lo2 - k2 - 1) + 1;   // smallest ky >= 0 with ky^2 >= lo2 - kx^2
-    const int yhi = isqrt_floor(hi2 - k2 < 0 ? 0 : hi2 - k2);
-    const int top = yhi < M ? yhi : M;
-    for (int ky = ylo; ky <= top; ++ky) h += wgt * energy(ky);
-    const int nlo = ylo > 1 ? ylo : 1;
-    for (int ky = -top; ky <= -nlo; ++ky) h += wgt * energy(ky);
+    bad += isfinite(w.x) && isfinite(w.y) ? 0 : 1;
   }
-  colhist[(size_t)kx * nbins + sh] = h;
+  if (bad) atomicAdd(badcount, bad);
+  __syncthreads();
+  const long long k2 = (long long)kx * kx;
+  for (int sh = threadIdx.x; sh < nbins; sh += 256) {
+    double h = 0.0;
+    const long long s2 = (long long)sh * sh;
+    const long long lo2 = sh == 0 ? 0 : s2 - sh + 1, hi2 = sh == 0 ? 0 : s2 + sh;   // range of m^2
+    if (hi2 >= k2) {
+      const int ylo = lo2 - k2 <= 0 ? 0 : isqrt_floor(lo2 - k2 - 1) + 1;   // smallest ky >= 0 with ky^2 >= lo2 - kx^2
+      const int yhi = isqrt_floor(hi2 - k2 < 0 ? 0 : hi2 - k2);
+      const int top = yhi < M ? yhi : M;
+      for (int ky = ylo; ky <= top; ++ky) h += wgt * en[ky];
+      const int nlo = ylo > 1 ? ylo : 1;
+      for (int ky = -top; ky <= -nlo; ++ky) h += wgt * en[ky + NK];
+    }
+    colhist[(size_t)kx * nbins + sh] = h;
+  }
 }
 
 template <typename T>

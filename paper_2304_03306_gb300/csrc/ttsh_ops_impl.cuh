@@ -170,7 +170,7 @@ static cudaError_t launch_col(int mode, const DomainDev& d, cudaStream_t s) {
 template <typename T, int N>
 static cudaError_t launch_spec(const DomainDev& d, int nbins, cudaStream_t s) {
   constexpr int H = N / 4 + 1;
-  spectrum_col_kernel<T, N><<<dim3((nbins + 127) / 128, H), 128, 0, s>>>(make_args<T>(d), nbins, d.colhist, d.bad);
+  spectrum_col_kernel<T, N><<<H, 256, 0, s>>>(make_args<T>(d), nbins, d.colhist, d.bad);
   return cudaGetLastError();
 }
 
