@@ -556,6 +556,19 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
 
   if constexpr (CL > 1) cluster_sync();   // every block's share is staged and visible
 
+  // In-place variants without staged mask rows: this thread's mask values travel in registers while
+  // the inverse transforms run (read where they are used, their latency was a third of the
+  // 2048^2 pass's stalls).  KI slots of two points per thread.
+  constexpr int KI = (R * L + NT - 1) / NT;
+  constexpr bool K_AHEAD = KIND == ROW_STEP && !Geo::SEPARATE && !Geo::STAGE_K && KI <= 8;
+  auto kload = [&](int e) { return reinterpret_cast<const cplx<T>*>(A.K + (size_t)y0 * N)[e]; };
+  cplx<T> kreg[K_AHEAD ? KI : 1];
+  if constexpr (K_AHEAD) {
+#pragma unroll
+    for (int i = 0; i < KI; ++i)
+      if (KI * NT <= R * L || tid + i * NT < R * L) kreg[i] = kload(tid + i * NT);
+  }
+
   // ---- inverse row transforms (C2R through an L-point complex transform) ----
   // The twiddle pre-pass that turns the half spectrum X of a real row into the L-point
   // complex input Z[k] = (X[k] + conj X[L-k]) + i conj(W_N^k) (X[k] - conj X[L-k]) is the
@@ -639,27 +652,45 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
     }
     fft_batch<T, L, PE, -1, NT, N, LP>(fw, FF * R, tw, stab, rhs);
   } else if constexpr (KIND == ROW_STEP) {
-    // the real-space terms in place; a recorded step also adds every point to the
-    // time-series sums as it reads it
+    // the real-space terms in place, a complex slot (points 2k and 2k + 1) at a time; a recorded
+    // step also adds every point to the time-series sums as it reads it
     auto terms = [&](auto rec_tag) {
       constexpr bool RS = decltype(rec_tag)::value;
       SeriesSums<T> ss;
       const T dx = (T)A.dx, cx = (T)A.cx, cy = (T)A.cy;
-      for (int e = tid; e < R * N; e += NT) {
-        const int r = e / N, x = e % N;
-        const T w = rl(0, r, x), vx = rl(1, r, x), vy = rl(2, r, x);
-        if constexpr (RS) ss.add(w, vx, vy, (T)(x - N / 2) * dx - cx, (T)(y0 + r - N / 2) * dx - cy);
-        T Kv;
-        if constexpr (Geo::STAGE_K) Kv = ks[e];
-        else Kv = A.K[(size_t)(y0 + r) * N + x];
+#pragma unroll
+      for (int i = 0; i < KI; ++i) {
+        const int e = tid + i * NT;
+        if (KI * NT > R * L && e >= R * L) break;
+        const int r = e / L, k = e % L;
+        cplx<T>* z = sm + r * LP + padi<PS>(k);
+        const cplx<T> w = z[0], vx = z[R * LP], vy = z[2 * R * LP];
+        cplx<T> Kv;
+        if constexpr (Geo::STAGE_K) Kv = reinterpret_cast<const cplx<T>*>(ks)[e];
+        else if constexpr (K_AHEAD) Kv = kreg[i];
+        else Kv = kload(e);
+        if constexpr (RS) {
+          const T px = (T)(2 * k - N / 2) * dx - cx, px1 = (T)(2 * k + 1 - N / 2) * dx - cx;
+          const T py = (T)(y0 + r - N / 2) * dx - cy;
+          ss.add(w.x, vx.x, vy.x, px, py);
+          ss.add(w.y, vx.y, vy.y, px1, py);
+        }
         // explicit fused multiply-adds: every kernel instantiation (single and batched)
         // rounds the same way
-        const T v2 = fma(vx, vx, vy * vy);
-        const T c1 = fma(-A.b, v2, -(A.gv * Kv));        // velocity terms: -b|v|^2 v - gamma_v K v = c1 v
-        const T lw = A.lam * w;                           // advection, conservative form
-        rl(0, r, x) = fma(c1, vx, lw * vy);
-        rl(1, r, x) = fma(c1, vy, -(lw * vx));
-        rl(2, r, x) = -(A.gw * Kv) * w;
+        auto point = [&](T wp, T vxp, T vyp, T Kp, T& f0, T& f1, T& f2) {
+          const T v2 = fma(vxp, vxp, vyp * vyp);
+          const T c1 = fma(-A.b, v2, -(A.gv * Kp));        // velocity terms: -b|v|^2 v - gamma_v K v = c1 v
+          const T lw = A.lam * wp;                           // advection, conservative form
+          f0 = fma(c1, vxp, lw * vyp);
+          f1 = fma(c1, vyp, -(lw * vxp));
+          f2 = -(A.gw * Kp) * wp;
+        };
+        cplx<T> f0, f1, f2;
+        point(w.x, vx.x, vy.x, Kv.x, f0.x, f1.x, f2.x);
+        point(w.y, vx.y, vy.y, Kv.y, f0.y, f1.y, f2.y);
+        z[0] = f0;
+        z[R * LP] = f1;
+        z[2 * R * LP] = f2;
       }
       if constexpr (RS) ss.template store<NT>(A, blk);
     };
