@@ -1067,11 +1067,11 @@ cudaError_t row_one(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup) {
   // One grid row a block where all of them fit at two (one for 512 points) an SM: a single A
   // tile then leaves room beside a column kernel's block, so that the row blocks are all in
   // place when the columns are done.  Beyond that as many blocks as fit walk over the rows:
-  // tensor memory (64 T of 512 columns each), shared memory, 32 warps of up to 128 registers.
+  // registers (row_blocks; tensor memory holds more) and shared memory.
   RowArgs r = a;
   r.tiles = a.Q <= 152LL * (T == 4 ? 1 : 2) || !row_has_mma(MODE) ? 1 : 2;
   const int smem = row_smem(MODE, TRAIN, f->n, r.tiles);
-  int per = T == 4 ? 1 : T == 2 ? 2 : 4;
+  int per = row_blocks(T, TRAIN);
   const int fit = (227 * 1024) / (smem + 2048);
   if (fit < per) per = fit < 1 ? 1 : fit;
   const long long cap = r.tiles == 1 && row_has_mma(MODE) ? a.Q : 152LL * per;

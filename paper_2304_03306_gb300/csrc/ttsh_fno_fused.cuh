@@ -97,10 +97,15 @@ __device__ __forceinline__ float4* row_piece(unsigned char* blk, int r, int i) {
   return reinterpret_cast<float4*>(blk + r * 128 + ((i ^ (r & 7)) << 4));
 }
 
+// Blocks per SM the row kernel is compiled for (registers) and launched with where a block walks
+// over several rows.
+__host__ __device__ constexpr int row_blocks(int T, bool train) { return T == 4 ? 1 : (train ? 4 : 6) / T; }
+
 template <int MODE, int T, bool TRAIN>
-__global__ void __launch_bounds__(128 * T, T == 4 ? 1 : TRAIN ? 2 : 3) row_layer_kernel(RowArgs a) {
+__global__ void __launch_bounds__(128 * T, row_blocks(T, TRAIN)) row_layer_kernel(RowArgs a) {
   constexpr int NT = 128 * T;
-  constexpr int TCOLS = 64 * T;   // per x tile: 32 columns for the channel mixing, 32 for the expansion
+  // per x tile: 32 columns for the channel mixing, 32 for the expansion
+  constexpr int TCOLS = row_has_mma(MODE) ? 64 * T : 32;
   extern __shared__ __align__(16) unsigned char row_dyn[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_base;
