@@ -99,12 +99,12 @@ __device__ __forceinline__ bool wait_count(const unsigned long long* ctr, unsign
 constexpr int kPersistMaxN = 512;
 
 // Float bodies in the forms with the least shared memory (the same values as the per-launch ones,
-// see CMP and LEAN): the stepper is bound by how many items an SM holds at once (30 KB a block
+// see CMP and LEAN): the stepper is bound by how many items an SM holds at once (28 KB a block
 // instead of 44).  48-domain sweep, 160 steps with the states read: 11.8 ms with the per-launch
-// forms at 5 blocks an SM; in place at 5 blocks 10.9, at 6 10.6, at 7 10.5 (spilling); with the
-// mask rows read from global memory as well 10.8.
+// forms at 5 blocks an SM; in place 10.9 at 5 and 10.6 at 6; with dense tiles and without unused
+// tables 10.2 at 6, 10.04 at 7, 10.08 at 8 (where registers spill).  Mask rows from global memory: slower.
 constexpr int kPersistCmp = 2;
-constexpr int kPersistBlocks = 6;   // resident blocks per SM the float kernel is compiled for
+constexpr int kPersistBlocks = 7;   // resident blocks per SM the float kernel is compiled for
 
 template <typename T, int N>
 struct PersistShape {
