@@ -235,10 +235,11 @@ struct TwTab {
       return cmul(hi[m >> SB], lo[m & (NLO - 1)]);
     }
   }
-  // Fill from the global table with cp.async (all threads of the block); the caller waits
-  // (cp_async_wait_all) and synchronises before the first use.
+  // Fill the first CNT entries from the global table with cp.async (all threads of the block);
+  // the caller waits (cp_async_wait_all) and synchronises before the first use.
+  template <int CNT = ENTRIES>
   __device__ __forceinline__ static TwTab fill(cplx<T>* sm, const cplx<T>* __restrict__ tw, int tid, int nt) {
-    for (int i = tid; i < ENTRIES; i += nt)
+    for (int i = tid; i < CNT; i += nt)
       cp_async<(int)sizeof(cplx<T>)>(sm + i, i < NLO ? tw + i : tw + (size_t)(i - NLO) * NLO);
     TwTab t;
     t.lo = sm;

@@ -172,8 +172,10 @@ struct RowGeo {
   static constexpr int NPL = FI;   // G planes read (field f comes from plane f)
   static constexpr int CB = (int)sizeof(cplx<T>);
   static constexpr int LPR = row_stride(LP, R, CB / 4);
-  static constexpr int TW_BYTES = align16(TwTab<T, N>::ENTRIES * CB) + StageTab<T, L, PE>::BYTES;
-  static constexpr int OFF_STAB = align16(TwTab<T, N>::ENTRIES * CB);
+  // W_N^k for the real-transform passes (k < L), and for the stages where they have no tables
+  static constexpr int TW_ENT = TwTab<T, N>::FULL && StageTab<T, L, PE>::USE ? L : TwTab<T, N>::ENTRIES;
+  static constexpr int TW_BYTES = align16(TW_ENT * CB) + StageTab<T, L, PE>::BYTES;
+  static constexpr int OFF_STAB = align16(TW_ENT * CB);
   // every region starts on a 16-byte boundary (16-byte cp.async destinations)
   static constexpr int BUF_BYTES = align16(F * R * LPR * CB);
   // staged G tile: plane f at OFF_GIN + f * GPS ([mx][r] inside a plane); planes start on
@@ -200,13 +202,15 @@ struct RowGeo {
   // four of them share a bank.  So without clusters (whose shares are exchanged in 16-byte
   // pieces) an even R gets one spare slot, where the padded tile still fits the budget that
   // decided the staging above.
+  // The spare slot costs 16-byte copies (8-byte ones then), which the in-place forms and the small
+  // grids feel more: 2048^2 compact pass 46.1 us dense, 50.3 padded; 48-domain sweep 10.2 and 10.4 ms.
   // Nor may the padding cost a block per SM (batched launches run several per SM): the
   // padded plan must leave as many blocks per SM as the dense one.
   static constexpr int RS_ODD = RS % 2 == 1 ? RS : RS + 1;
   static constexpr int PAD_EXTRA = STAGE_G ? NPL * (align128(HC * RS_ODD * CB) - align128(HC * RS * CB)) : 0;
   static constexpr int SMEM_DENSE = align128(TW_BYTES + BUF_BYTES) + (STAGE_G ? GIN_DENSE : 0) +
       (STAGE_K ? KS_BYTES : 0) + RED_BYTES + (SEPARATE ? BUF_BYTES : 0) + 128;
-  static constexpr bool PAD_G = CL == 1 && STAGE_G && RS_ODD != RS &&
+  static constexpr bool PAD_G = CL == 1 && CMP == 0 && N >= 512 && STAGE_G && RS_ODD != RS &&
       TW_BYTES + (SEPARATE ? 2 : 1) * BUF_BYTES + GIN_DENSE + PAD_EXTRA + (STAGE_K ? KS_BYTES : 0) + RED_BYTES <=
           kSmemLimit &&
       smem_blocks_per_sm(SMEM_DENSE + PAD_EXTRA) == smem_blocks_per_sm(SMEM_DENSE);
@@ -251,8 +255,9 @@ struct ColGeo {
                          : (MODE == COL_MASK || MODE == COL_ADDW) ? 1 : 0;
   static constexpr int NI = MODE == COL_MASK ? 1 : MODE == COL_DIV ? 0 : 3;
   static constexpr int CB = (int)sizeof(cplx<T>);
-  static constexpr int TW_BYTES = align16(TwTab<T, N>::ENTRIES * CB) + StageTab<T, N, PE>::BYTES;
-  static constexpr int OFF_STAB = align16(TwTab<T, N>::ENTRIES * CB);
+  static constexpr int TW_ENT = StageTab<T, N, PE>::USE ? 0 : TwTab<T, N>::ENTRIES;   // stages without tables
+  static constexpr int TW_BYTES = align16(TW_ENT * CB) + StageTab<T, N, PE>::BYTES;
+  static constexpr int OFF_STAB = align16(TW_ENT * CB);
   static constexpr int ACC_BYTES = align16(NK * CB);
   static constexpr int WS_BYTES = (MODE == COL_STEP || MODE == COL_ADDW || MODE == COL_DIV) ? align16(NK * CB) : 0;
   static constexpr int FIXED = TW_BYTES + ACC_BYTES + WS_BYTES + 64;
@@ -505,7 +510,7 @@ __device__ __forceinline__ void row_body(const Args<T>& A, int blk, unsigned cha
 
   // ---- stage: twiddles and the K rows (inputs no previous kernel writes), then, once the
   // previous kernel has finished, the G tile (R consecutive y of every stored column) ----
-  const TwTab<T, N> tw = TwTab<T, N>::fill(reinterpret_cast<cplx<T>*>(smem_raw), A.tw, tid, NT);
+  const TwTab<T, N> tw = TwTab<T, N>::template fill<Geo::TW_ENT>(reinterpret_cast<cplx<T>*>(smem_raw), A.tw, tid, NT);
   cplx<T>* stab = reinterpret_cast<cplx<T>*>(smem_raw + Geo::OFF_STAB);
   StageTab<T, L, PE>::template fill<N>(stab, A.tw, tid, NT);
   if constexpr (Geo::STAGE_K) {
@@ -843,7 +848,7 @@ __device__ __forceinline__ void col_body(const Args<T>& A, int kx, unsigned char
   const T fwdN = (T)0.5 / (T)N;   // the row pass leaves twice its transform
   constexpr int CB = Geo::CB;
 
-  const TwTab<T, N> tw = TwTab<T, N>::fill(reinterpret_cast<cplx<T>*>(smem_raw), A.tw, tid, NT);
+  const TwTab<T, N> tw = TwTab<T, N>::template fill<Geo::TW_ENT>(reinterpret_cast<cplx<T>*>(smem_raw), A.tw, tid, NT);
   cplx<T>* stab = reinterpret_cast<cplx<T>*>(smem_raw + Geo::OFF_STAB);
   StageTab<T, N, PE>::template fill<N>(stab, A.tw, tid, NT);
   griddep_wait();   // everything below reads what the previous kernel wrote
@@ -1094,18 +1099,29 @@ row_io_kernel(Args<T> A, FieldIo io) {
   row_body<T, N, KIND, R, PEV>(A, blockIdx.x, smem_base128(smem_raw), nullptr, &io);
 }
 
+// The column step takes the lean form where that lets an SM hold more blocks and the grid has them
+// (2048^2 float, 513 blocks: two an SM instead of one, 28.8 -> 24.6 us).
+constexpr int kSms = 152;
 template <typename T, int N, int MODE, int PEV>
-__global__ void __launch_bounds__(ColGeo<T, N, MODE, PEV>::NT)
+__host__ __device__ constexpr int col_lean() {
+  using Dense = ColGeo<T, N, MODE, PEV, 0>;
+  using Lean = ColGeo<T, N, MODE, PEV, 1>;
+  return MODE == COL_STEP && Dense::BULK && smem_blocks_per_sm(Lean::SMEM) > smem_blocks_per_sm(Dense::SMEM) &&
+         Dense::H > kSms * smem_blocks_per_sm(Dense::SMEM);
+}
+
+template <typename T, int N, int MODE, int PEV, int LEAN = 0>
+__global__ void __launch_bounds__(ColGeo<T, N, MODE, PEV, LEAN>::NT)
 col_kernel(Args<T> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (MODE == COL_STEP) {
-    if (blockIdx.x == ColGeo<T, N, MODE, PEV>::H) {   // launched only for a recorded step
-      static_assert(ColGeo<T, N, MODE, PEV>::NT >= 32, "the sample block needs a whole warp 0");
+    if (blockIdx.x == ColGeo<T, N, MODE, PEV, LEAN>::H) {   // launched only for a recorded step
+      static_assert(ColGeo<T, N, MODE, PEV, LEAN>::NT >= 32, "the sample block needs a whole warp 0");
       record_sample(A);
       return;
     }
   }
-  col_body<T, N, MODE, PEV>(A, blockIdx.x, smem_raw);
+  col_body<T, N, MODE, PEV, LEAN>(A, blockIdx.x, smem_raw);
 }
 
 // Batched variants: blockIdx.y selects the domain, whose arguments live in a device array.

@@ -111,14 +111,15 @@ static cudaError_t launch_row_kind(const DomainDev& d, cudaStream_t s) {
 // again steps on bit for bit: the prologue makes the same row inputs as the step's column pass)
 template <typename T, int N, int MODE, int PE = default_step_col_pe<T, N>()>
 static cudaError_t launch_col_mode(const DomainDev& d, cudaStream_t s) {
-  using Geo = ColGeo<T, N, MODE, PE>;
+  constexpr int LEAN = col_lean<T, N, MODE, PE>();
+  using Geo = ColGeo<T, N, MODE, PE, LEAN>;
   static std::atomic<int> done{0};
-  cudaError_t e = set_smem(col_kernel<T, N, MODE, PE>, cmax(Geo::SMEM, kSpreadSmem), done);
+  cudaError_t e = set_smem(col_kernel<T, N, MODE, PE, LEAN>, cmax(Geo::SMEM, kSpreadSmem), done);
   if (e != cudaSuccess) return e;
   // a recorded step adds one block that finishes the time-series sample
   const int extra = (MODE == COL_STEP && d.rec != nullptr) ? 1 : 0;
   const bool pdl = MODE == COL_STEP && step_pdl<N>(d);
-  return launch_k(col_kernel<T, N, MODE, PE>, Geo::H + extra, Geo::NT, launch_smem(Geo::SMEM, Geo::H + extra, pdl), s,
+  return launch_k(col_kernel<T, N, MODE, PE, LEAN>, Geo::H + extra, Geo::NT, launch_smem(Geo::SMEM, Geo::H + extra, pdl), s,
                   pdl, 1, make_args<T>(d));
 }
 
@@ -296,8 +297,9 @@ static SizeOps make_ops() {
   o.alone_row = find_shape(o.row_step, o.n_row_variants, F32 ? (N <= 256 ? 2 : 4) : (N <= 256 ? 1 : 2),
                            F32 ? (N <= 256 ? 8 : 16) : (N <= 256 ? 4 : 8), 0);
   o.alone_col = find_shape(o.col_step, o.n_col_variants, 1, F32 || N <= 256 ? 4 : 8, 0);
-  // 2048^2 float starts with the compact two-row pass (50.8 us; the plain one 58.1)
-  o.start_row = F32 && N == 2048 ? find_shape(o.row_step, o.n_row_variants, 2, 16, 1) : 0;
+  // 2048^2 and 4096^2 float start with the compact two-row pass (46.1 and 219.5 us; the plain ones
+  // 57.0 and 232)
+  o.start_row = F32 && (N == 2048 || N == 4096) ? find_shape(o.row_step, o.n_row_variants, 2, 16, 1) : 0;
   return o;
 }
 
