@@ -1320,8 +1320,9 @@ ttsh_status ttsh_autotune(ttsh_domain* d, int32_t iters, int32_t* plan) {
   if ((st = restore_state(d)) != TTSH_OK) return st;
   if ((st = ttsh_set_plan(d, br, bc)) != TTSH_OK) return st;
   // launch mode: whole steps (row then column pass) with and without programmatic
-  // dependent launch; keep the faster
-  double t_mode[2];
+  // dependent launch; keep the faster (up to 512^2 steps overlap in either mode)
+  double t_mode[2] = {0, 0};
+  if (d->n <= ttsh::kPdlMaxN) return (st = ttsh_set_launch_mode(d, btma << 1)) != TTSH_OK ? st : ttsh_get_plan(d, plan);
   for (int pdl = 0; pdl < 2; ++pdl) {
     if ((st = ttsh_set_launch_mode(d, pdl | (btma << 1))) != TTSH_OK) return st;
     if ((st = save_state(d)) != TTSH_OK) return st;

@@ -77,6 +77,7 @@ struct StepVariant {
 };
 
 constexpr int kMaxBatchN = 1024;
+constexpr int kPdlMaxN = 512;   // grids up to here: captured steps overlap in any launch mode
 
 constexpr int kMaxVariants = 12;
 

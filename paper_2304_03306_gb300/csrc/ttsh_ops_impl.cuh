@@ -47,7 +47,6 @@ static int launch_smem(int smem, int grid, bool pdl) {
 // 26.8 -> 23.4, 2048^2 87.2 -> 81.9); in a graph it saves 0.5 us of a small grid's pass (256^2
 // 8.47 -> 7.34 us a step, 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1) but costs at 1024^2
 // (22.7 -> 23.8) and does nothing beyond.
-constexpr int kPdlMaxN = 512;
 template <int N>
 static bool step_pdl(const DomainDev& d) { return !d.whole && (d.pdl || !d.captured || N <= kPdlMaxN); }
 
