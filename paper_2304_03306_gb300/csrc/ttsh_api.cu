@@ -759,12 +759,16 @@ struct ttsh_batch {
   void* pitems = nullptr;              // device work-item list of one step
   void* ptest = nullptr;               // one-item list of ttsh_batch_test_stalled_wait
   unsigned long long* pctl = nullptr;  // device control block: 2 + 2 ndom counters
-  int pips = 0, pgrid = 0;
+  int pips = 0, pgrid = 0, plean = 0;
 };
 
 namespace {
 
 constexpr int kBatchGraphLen = 32;
+// Items a step from which the persistent stepper's lean form pays (us a step, per-launch and lean
+// form: 12 domains, 1292 items 19.9 and 23.8; 26 domains, 3418 items 30.9 and 32.7; 32 domains,
+// 4128 items 37.1 and 33.6; 48 domains, 6448 items 57.7 and 50.3)
+constexpr int kLeanItems = 3700;
 
 ttsh_status batch_group_steps(BatchGroup& g, int nsteps, cudaStream_t s) {
   const int nd = (int)g.doms.size();
@@ -1470,6 +1474,7 @@ ttsh_status ttsh_batch_create(ttsh_domain* const* domains, int32_t ndom, void* s
             }
           }
       b->pips = (int)(items.size() / 4);
+      b->plean = b->pips > kLeanItems;
       static_assert(sizeof(int) * 4 == 16, "work item layout");
       cudaError_t pe = b->pops.item_bytes == 16 ? cudaSuccess : cudaErrorInvalidValue;
       if (pe == cudaSuccess) pe = cudaMalloc(&b->pdoms, dt.size());
@@ -1477,7 +1482,7 @@ ttsh_status ttsh_batch_create(ttsh_domain* const* domains, int32_t ndom, void* s
       if (pe == cudaSuccess) pe = cudaMalloc(&b->pctl, (2 + 2 * (size_t)nd) * sizeof(unsigned long long));
       if (pe == cudaSuccess) pe = cudaMemcpy(b->pdoms, dt.data(), dt.size(), cudaMemcpyHostToDevice);
       if (pe == cudaSuccess) pe = cudaMemcpy(b->pitems, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice);
-      if (pe == cudaSuccess) pe = b->pops.prepare(&b->pgrid);
+      if (pe == cudaSuccess) pe = b->pops.prepare(b->plean, &b->pgrid);
       if (pe != cudaSuccess) return cleanup(cuda_fail(pe, "persistent batch set-up"));
       b->can_persist = true;
       b->persistent = true;
@@ -1515,7 +1520,7 @@ ttsh_status ttsh_batch_step(ttsh_batch* b, int64_t nsteps) {
     if (nsteps > 0) {
       const size_t ctl_bytes = (2 + 2 * b->all.size()) * sizeof(unsigned long long);
       TTSH_CUDA(cudaMemsetAsync(b->pctl, 0, ctl_bytes, b->stream), "persistent batch reset");
-      TTSH_CUDA(b->pops.launch(b->pdoms, b->pitems, b->pips, (long long)nsteps, b->pctl, b->pgrid, ttsh::kWaitLimitNs,
+      TTSH_CUDA(b->pops.launch(b->plean, b->pdoms, b->pitems, b->pips, (long long)nsteps, b->pctl, b->pgrid, ttsh::kWaitLimitNs,
                                b->stream),
                 "persistent batch launch");
     }
@@ -1585,7 +1590,7 @@ ttsh_status ttsh_batch_test_stalled_wait(ttsh_batch* b, double seconds) {
   }
   const size_t ctl_bytes = (2 + 2 * b->all.size()) * sizeof(unsigned long long);
   TTSH_CUDA(cudaMemsetAsync(b->pctl, 0, ctl_bytes, b->stream), "persistent batch reset");
-  TTSH_CUDA(b->pops.launch(b->pdoms, b->ptest, 1, 1, b->pctl, 1, (unsigned long long)(seconds * 1e9), b->stream),
+  TTSH_CUDA(b->pops.launch(b->plean, b->pdoms, b->ptest, 1, 1, b->pctl, 1, (unsigned long long)(seconds * 1e9), b->stream),
             "stalled persistent launch");
   return TTSH_OK;
 }

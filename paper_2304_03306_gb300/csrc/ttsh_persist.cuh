@@ -98,31 +98,32 @@ __device__ __forceinline__ bool wait_count(const unsigned long long* ctr, unsign
 // Sizes the persistent kernel holds (the batched sweeps' grids and smaller).
 constexpr int kPersistMaxN = 512;
 
-// Float bodies in the forms with the least shared memory (the same values as the per-launch ones,
-// see CMP and LEAN): the stepper is bound by how many items an SM holds at once (28 KB a block
-// instead of 44).  48-domain sweep, 160 steps with the states read: 11.8 ms with the per-launch
-// forms at 5 blocks an SM; in place 10.9 at 5 and 10.6 at 6; with dense tiles and without unused
-// tables 10.2 at 6, 10.04 at 7, 10.08 at 8 (where registers spill).  Mask rows from global memory: slower.
-constexpr int kPersistCmp = 2;
-constexpr int kPersistBlocks = 7;   // resident blocks per SM the float kernel is compiled for
+// Two forms of the float kernel (the same values, see CMP and LEAN).  LEAN_FORM: the bodies with the
+// least shared memory (28 KB a block instead of 42), seven blocks an SM: what bounds a batch with many
+// items is how many of them an SM holds at once.  Otherwise the per-launch bodies, whose chain of
+// phases is shorter, five blocks an SM: a batch with few items waits for each item.
+// 48-domain sweep (6448 items a step), 160 steps with the states read: 11.8 ms in the per-launch
+// forms; lean 10.9 at 5 blocks, 10.2 at 6, 10.04 at 7, 10.08 at 8 (where registers spill).
+template <typename T>
+__host__ __device__ constexpr int persist_blocks(bool lean) { return sizeof(T) == 4 ? (lean ? 7 : 5) : 2; }
 
-template <typename T, int N>
+template <typename T, int N, bool LF>
 struct PersistShape {
   static constexpr int R = default_step_rows<T, N>();
   static constexpr int RPE = default_step_row_pe<T, N>();
   static constexpr int CPE = default_step_col_pe<T, N>();
-  static constexpr int CMP = sizeof(T) == 4 ? kPersistCmp : 0;
-  static constexpr int LEAN = sizeof(T) == 4 ? 1 : 0;
+  static constexpr int CMP = sizeof(T) == 4 && LF ? 2 : 0;
+  static constexpr int LEAN = sizeof(T) == 4 && LF ? 1 : 0;
   using RG = RowGeo<T, N, ROW_STEP, R, RPE, 1, CMP>;
   using CG = ColGeo<T, N, COL_STEP, CPE, LEAN>;
   static constexpr int NT = cmax(RG::NT, CG::NT);
   static constexpr int SMEM = cmax(RG::SMEM, CG::SMEM);
 };
 
-template <typename T>
+template <typename T, bool LF>
 struct PersistLimits {
   template <int N>
-  using S = PersistShape<T, N>;
+  using S = PersistShape<T, N, LF>;
   static constexpr int NT = cmax(cmax(cmax(S<16>::NT, S<32>::NT), cmax(S<64>::NT, S<128>::NT)),
                                  cmax(S<256>::NT, S<512>::NT));
   static constexpr int SMEM = cmax(cmax(cmax(S<16>::SMEM, S<32>::SMEM), cmax(S<64>::SMEM, S<128>::SMEM)),
@@ -134,26 +135,26 @@ struct PersistLimits {
 // The argument block is copied out of the domain table first (as the per-launch batched
 // kernels do), so the body's constants live in registers rather than being reloaded from
 // global memory after every store.
-template <typename T, int N>
+template <typename T, int N, bool LF>
 __device__ __noinline__ void persist_row(const Args<T>& Ag, int blk, unsigned char* smem) {
-  using S = PersistShape<T, N>;
+  using S = PersistShape<T, N, LF>;
   if (threadIdx.x < S::RG::NT) {
     const Args<T> A = Ag;
     row_body<T, N, ROW_STEP, S::R, S::RPE, 1, S::CMP, false>(A, blk, smem, nullptr);
   }
 }
-template <typename T, int N>
+template <typename T, int N, bool LF>
 __device__ __noinline__ void persist_col(const Args<T>& Ag, int blk, unsigned char* smem) {
-  using S = PersistShape<T, N>;
+  using S = PersistShape<T, N, LF>;
   if (threadIdx.x < S::CG::NT) {
     const Args<T> A = Ag;
     col_body<T, N, COL_STEP, S::CPE, S::LEAN>(A, blk, smem);
   }
 }
-template <typename T, int N>
+template <typename T, int N, bool LF>
 __device__ __forceinline__ void persist_item(const Args<T>& A, int phase, int blk, unsigned char* smem) {
-  if (phase == 0) persist_row<T, N>(A, blk, smem);
-  else persist_col<T, N>(A, blk, smem);
+  if (phase == 0) persist_row<T, N, LF>(A, blk, smem);
+  else persist_col<T, N, LF>(A, blk, smem);
 }
 
 // Requirement of item it of step st: the counter it waits on and the count it needs.
@@ -177,11 +178,11 @@ __device__ __forceinline__ void item_need(const PDomain<T>* doms, const PItem& i
 // first, then waits for g' (which may depend on g) and publishes it behind one more barrier.
 // Published items alternate between two slots, so a slot is never rewritten while a thread
 // may still read it.
-template <typename T>
-__global__ void __launch_bounds__(PersistLimits<T>::NT + 32, sizeof(T) == 4 ? kPersistBlocks : 2)
+template <typename T, bool LF>
+__global__ void __launch_bounds__(PersistLimits<T, LF>::NT + 32, persist_blocks<T>(LF))
 persistent_step_kernel(const PDomain<T>* __restrict__ doms, const PItem* __restrict__ items, int ips,
                        long long nsteps, unsigned long long* __restrict__ ctl, unsigned long long limit_ns) {
-  constexpr int NB = PersistLimits<T>::NT;
+  constexpr int NB = PersistLimits<T, LF>::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_base128(smem_raw);
   __shared__ long long s_item[2];
@@ -237,12 +238,12 @@ persistent_step_kernel(const PDomain<T>* __restrict__ doms, const PItem* __restr
     if (threadIdx.x < NB) {
       const Args<T>& A = s_st[slot].A;
       switch (s_st[slot].n) {
-        case 16: persist_item<T, 16>(A, it.phase, it.blk, smem); break;
-        case 32: persist_item<T, 32>(A, it.phase, it.blk, smem); break;
-        case 64: persist_item<T, 64>(A, it.phase, it.blk, smem); break;
-        case 128: persist_item<T, 128>(A, it.phase, it.blk, smem); break;
-        case 256: persist_item<T, 256>(A, it.phase, it.blk, smem); break;
-        case 512: persist_item<T, 512>(A, it.phase, it.blk, smem); break;
+        case 16: persist_item<T, 16, LF>(A, it.phase, it.blk, smem); break;
+        case 32: persist_item<T, 32, LF>(A, it.phase, it.blk, smem); break;
+        case 64: persist_item<T, 64, LF>(A, it.phase, it.blk, smem); break;
+        case 128: persist_item<T, 128, LF>(A, it.phase, it.blk, smem); break;
+        case 256: persist_item<T, 256, LF>(A, it.phase, it.blk, smem); break;
+        case 512: persist_item<T, 512, LF>(A, it.phase, it.blk, smem); break;
         default: break;
       }
       if (threadIdx.x == 0) s_body_done = g;   // a hint for the control lane's poll
