@@ -911,7 +911,7 @@ ttsh_status ttsh_create_domain(const uint8_t* mask, const ttsh_params* p, void* 
   d->graph = nullptr;
   d->graph_len = 0;
   d->rv = ops.start_row;
-  d->cv = 0;
+  d->cv = ops.start_col;
   d->lay = layout_for(d->n, d->elt);
   d->owns_ws = workspace == nullptr;
   d->ws = workspace;

@@ -122,12 +122,12 @@ __host__ __device__ constexpr int default_col_pe() { return sizeof(T) == 4 ? (N 
 // 3.7 us per row pass - but slower in a batch, where twice the blocks pay their fixed costs
 // twice: 53.0 against 49.9 us per step of the 48-domain sweep; so they stay autotuner
 // choices.)
-// The larger grids start with the shapes measured fastest: 4096^2 two rows (238 us; one row 327),
-// 1024^2 a 16-point column pass (7.8 us; 8-point 8.1).  Double up to 256^2: one row and 4 points per thread in both passes
+// 1024^2 float: a 16-point column pass (7.8 us; 8-point 8.1), not first in its list (an index of
+// a saved plan keeps its shape).  Double up to 256^2: one row and 4 points per thread in both passes
 // (64^2 27 -> 17 us a step, 256^2 41 -> 35), in batches as well.
 template <typename T, int N>
 __host__ __device__ constexpr int default_step_rows() {
-  return sizeof(T) == 4 ? (N == 512 || N == 4096 ? 2 : default_rows<T, N>()) : (N <= 256 ? 1 : default_rows<T, N>());
+  return sizeof(T) == 4 ? (N == 512 ? 2 : default_rows<T, N>()) : (N <= 256 ? 1 : default_rows<T, N>());
 }
 template <typename T, int N>
 __host__ __device__ constexpr int default_step_row_pe() {

@@ -89,7 +89,7 @@ struct SizeOps {
   int n_row_variants, n_col_variants;           // entry 0: the batches' tile shape
   StepVariant row_step[kMaxVariants];
   StepVariant col_step[kMaxVariants];
-  int start_row;              // row variant a domain starts with (the column variant is 0)
+  int start_row, start_col;   // variants a domain starts with
   int alone_row, alone_col;   // fastest shapes of one domain stepped by itself (ttsh_step_noalloc)
   int args_bytes;                                    // size of one kernel argument block
   void (*pack_args)(const DomainDev&, void* dst);    // host copy of a domain's argument block

@@ -262,6 +262,7 @@ static SizeOps make_ops() {
   o.args_bytes = (int)sizeof(Args<T>);
   o.pack_args = &pack_args<T>;
   add_row_variant<T, N, default_step_rows<T, N>(), default_step_row_pe<T, N>(), default_row_cluster<T, N>()>(o);
+  if constexpr (sizeof(T) == 4 && N == 1024) add_col_variant<T, N, default_col_pe<T, N>()>(o);
   add_col_variant<T, N, default_step_col_pe<T, N>()>(o);
   if constexpr (sizeof(T) == 4) {
     add_row_variant<T, N, 4, 16>(o);
@@ -299,6 +300,7 @@ static SizeOps make_ops() {
   // 2048^2 and 4096^2 float start with the compact two-row pass (46.1 and 219.5 us; the plain ones
   // 57.0 and 232)
   o.start_row = F32 && (N == 2048 || N == 4096) ? find_shape(o.row_step, o.n_row_variants, 2, 16, 1) : 0;
+  o.start_col = F32 && N == 1024 ? find_shape(o.col_step, o.n_col_variants, 1, default_step_col_pe<T, N>(), 0) : 0;
   return o;
 }
 
