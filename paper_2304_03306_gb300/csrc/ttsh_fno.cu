@@ -7,14 +7,12 @@
 // and ky in {0..m-1} U {n-m..n-1}, one complex C x C matrix per kept mode.
 //
 // Arithmetic: learned weights are held as FP32 master copies and used in BF16 by the kernels;
-// every product accumulates in FP32.  The channel-mixing layers (h W, and dz W^T in the
-// backward pass) run on the 5th-generation tensor cores (tcgen05.mma BF16 -> FP32 in tensor
-// memory, fused bias / residual / GELU epilogue).  The transforms restricted to the kept
-// modes are exact DFT matrices (2m x n per row and per column, cheaper than a full FFT when
-// m << n).  The row transforms (onto the kept kx and back, and their adjoints in the backward
-// pass) run on the tensor cores as well (BF16 operands, FP32 accumulation); the column
-// transforms along y with the per-mode complex mixing run in dedicated FP32 kernels that read
-// BF16 weights.
+// every product accumulates in FP32.  The transforms restricted to the kept modes are exact DFT
+// matrices (2m x n per row and per column, cheaper than a full FFT when m << n).  For n % 16 == 0,
+// n <= 512 and an even number of modes <= 16 a layer is two kernels (ttsh_fno_fused.cuh: row
+// transforms and channel mixing on the tensor cores, column transforms and per-mode mixing in
+// FP32 clusters); the kernels here with one operation each serve the other shapes, in the same
+// order of sums.
 // Gradients use fixed-order partial sums, so repeated calls give identical bits.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
