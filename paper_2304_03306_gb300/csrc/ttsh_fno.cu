@@ -1047,12 +1047,26 @@ cudaError_t launch_layer(void (*k)(A), dim3 grid, int block, int smem, cudaStrea
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 
-// Shared-memory limit, and the largest carve-out: row and column kernels of one pass share the
-// SMs, so that a kernel's blocks are in place, their constant operands staged, when the one
-// before it ends.
+// Allows a kernel all the dynamic shared memory the device leaves beside its static one.  Networks of
+// every shape launch the same kernels with sizes of their own, and the attribute replaces the
+// one before it: this is the same value whichever network sets it, in whatever order or thread.
 template <typename K>
-cudaError_t layer_attributes(K k, int smem) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+cudaError_t allow_smem(K k) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes at;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, k);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+  return e;
+}
+
+// The same, and the largest carve-out: row and column kernels of one pass share the SMs, so that a
+// kernel's blocks are in place, their constant operands staged, when the one before it ends.
+template <typename K>
+cudaError_t layer_attributes(K k) {
+  cudaError_t e = allow_smem(k);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   return e;
@@ -1061,7 +1075,7 @@ cudaError_t layer_attributes(K k, int smem) {
 template <int MODE, int T, bool TRAIN>
 cudaError_t row_one(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup) {
   auto k = &row_layer_kernel<MODE, T, TRAIN>;
-  if (setup) return layer_attributes(k, row_smem(MODE, TRAIN, f->n, 2));
+  if (setup) return layer_attributes(k);
   // One grid row a block where all of them fit at two (one for 512 points) an SM: a single A
   // tile then leaves room beside a column kernel's block, so that the row blocks are all in
   // place when the columns are done.  Beyond that as many blocks as fit walk over the rows:
@@ -1086,11 +1100,11 @@ cudaError_t run_row(ttsh_fno* f, const RowArgs& a, bool pdl, bool setup = false)
 template <bool ADJ>
 cudaError_t run_column(ttsh_fno* f, const ColArgs& a, int B, bool pdl, bool setup = false) {
   auto k = &column_layer_kernel<ADJ>;
+  if (setup) return layer_attributes(k);
   const int pieces = f->n / col_piece(f->n), two = pieces < 2 ? pieces : 2;
   ColArgs c = a;
   c.ring = CS * f->m * B <= 152 && pieces <= 4 ? pieces : two;   // (up to 256^2: 64 KB)
   const int smem = col_smem(f->n, f->m, c.ring, ADJ);
-  if (setup) return layer_attributes(k, col_smem(f->n, f->m, pieces <= 4 ? pieces : 2, ADJ));
   return launch_layer(k, dim3((unsigned)(CS * f->m), (unsigned)B), kColThreads, smem, f->stream, pdl, CS, c);
 }
 
@@ -1112,7 +1126,7 @@ cudaError_t fused_setup(ttsh_fno* f) {
 cudaError_t wgrad_setup() {
   cudaError_t e = cudaSuccess;
   auto wg = [&](auto k) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+    if (e == cudaSuccess) e = allow_smem(k);
   };
   wg(&wgrad_kernel<WA_RAW, WD_ONE>);
   wg(&wgrad_kernel<WA_RAW, WD_OUTER>);
@@ -1556,12 +1570,9 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
     e = fused_setup(f);
     if (e != cudaSuccess) return cleanup(fno_cuda(e, "layer kernel attribute"));
   } else if (f->fused_columns) {
-    e = cudaFuncSetAttribute(column_fwd_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             column_fwd_mix_smem(n));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(row_dft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, row_dft_smem(n, m));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(row_idft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, row_idft_smem(n, m));
+    e = allow_smem(&column_fwd_mix_kernel);
+    if (e == cudaSuccess) e = allow_smem(&row_dft_kernel);
+    if (e == cudaSuccess) e = allow_smem(&row_idft_kernel);
     if (e != cudaSuccess) return cleanup(fno_cuda(e, "column kernel attribute"));
   }
   // DFT matrices on the kept modes
@@ -1619,7 +1630,7 @@ ttsh_status ttsh_fno_create(const ttsh_fno_config* cfg, uint64_t seed, void* str
       e = cudaMemcpy(bdst[i], bsrc[i]->data(), bsrc[i]->size() * 2, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cleanup(fno_cuda(e, "DFT matrices"));
     if (f->tc_rows && !f->fused) {
-      e = cudaFuncSetAttribute(xcontract_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, xcontract_smem(n));
+      e = allow_smem(&xcontract_tc_kernel);
       if (e != cudaSuccess) return cleanup(fno_cuda(e, "row contraction attribute"));
     }
   }
