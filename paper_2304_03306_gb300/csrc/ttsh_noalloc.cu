@@ -34,7 +34,8 @@
 
 namespace {
 
-constexpr int kNoAllocMaxN = 512;
+constexpr int kNoAllocMaxN = ttsh::kAloneMaxN;
+static_assert(kNoAllocMaxN == 512, "the limit that ttsh.h states");
 constexpr size_t kMaxH = kNoAllocMaxN / 4 + 1;
 constexpr size_t kGBytes = 3 * kMaxH * kNoAllocMaxN * 2 * sizeof(double);
 constexpr size_t kRBytes = 3 * kMaxH * kNoAllocMaxN * 2 * sizeof(double);
@@ -151,7 +152,7 @@ extern "C" ttsh_status ttsh_step_noalloc(const ttsh_params* p, const void* K, vo
   d.n = p->n;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // rebuild the row-pass inputs from the caller's state, then step
-  e = ops.col(ttsh::K_COL_PROLOGUE, d, s);
+  e = ops.alone_prologue(d, s);
   for (int64_t i = 0; i < nsteps && e == cudaSuccess; ++i) {
     e = ops.row_step[ops.alone_row].fn(d, s);
     if (e == cudaSuccess) e = ops.col_step[ops.alone_col].fn(d, s);

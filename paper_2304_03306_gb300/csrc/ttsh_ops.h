@@ -79,6 +79,8 @@ struct StepVariant {
 constexpr int kMaxBatchN = 1024;
 constexpr int kPdlMaxN = 512;   // grids up to here: captured steps overlap in any launch mode
 
+constexpr int kAloneMaxN = 512;   // largest grid of ttsh_step_noalloc
+
 constexpr int kMaxVariants = 12;
 
 struct SizeOps {
@@ -91,6 +93,7 @@ struct SizeOps {
   StepVariant col_step[kMaxVariants];
   int start_row, start_col;   // variants a domain starts with
   int alone_row, alone_col;   // fastest shapes of one domain stepped by itself (ttsh_step_noalloc)
+  StepFn alone_prologue;      // row inputs from the state, in alone_col's shape (null above kAloneMaxN)
   int args_bytes;                                    // size of one kernel argument block
   void (*pack_args)(const DomainDev&, void* dst);    // host copy of a domain's argument block
 };

@@ -294,9 +294,15 @@ static SizeOps make_ops() {
   // more blocks and halve the butterflies of a thread's chain (float, us a step: 64^2 6.3 -> 4.9,
   // 256^2 7.3 -> 6.0; double 64^2 26 -> 17, 256^2 40 -> 35).
   constexpr bool F32 = sizeof(T) == 4;
+  // The prologue that starts a call has the column step's shape: it rounds the row inputs as the step
+  // it stands for would have, so that calls of k steps and one of 2k leave the same bits.  (Grids
+  // below 64^2 have one column variant.)
+  constexpr int ALONE_PE = N < 64 ? default_step_col_pe<T, N>() : F32 || N <= 256 ? 4 : 8;
   o.alone_row = find_shape(o.row_step, o.n_row_variants, F32 ? (N <= 256 ? 2 : 4) : (N <= 256 ? 1 : 2),
                            F32 ? (N <= 256 ? 8 : 16) : (N <= 256 ? 4 : 8), 0);
-  o.alone_col = find_shape(o.col_step, o.n_col_variants, 1, F32 || N <= 256 ? 4 : 8, 0);
+  o.alone_col = find_shape(o.col_step, o.n_col_variants, 1, cmin(ALONE_PE, N), 0);
+  o.alone_prologue = nullptr;
+  if constexpr (N <= kAloneMaxN) o.alone_prologue = &launch_col_mode<T, N, COL_PROLOGUE, ALONE_PE>;
   // 2048^2 and 4096^2 float start with the compact two-row pass (46.1 and 219.5 us; the plain ones
   // 57.0 and 232)
   o.start_row = F32 && (N == 2048 || N == 4096) ? find_shape(o.row_step, o.n_row_variants, 2, 16, 1) : 0;
