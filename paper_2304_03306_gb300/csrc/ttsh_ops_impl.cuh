@@ -208,14 +208,15 @@ static void pack_args(const DomainDev& d, void* dst) {
   memcpy(dst, &a, sizeof(a));
 }
 
+// (again: a shape that is in the list already gets this index as well)
 template <typename T, int N, int R, int PE, int CL = 1, int CMP = 0>
-static void add_row_variant(SizeOps& o) {
+static void add_row_variant(SizeOps& o, bool again = false) {
   if constexpr (RowGeo<T, N, ROW_STEP, R, PE, CL, CMP>::VALID &&
                 (N >= 64 || (R == default_step_rows<T, N>() && PE == default_step_row_pe<T, N>() && CL == 1 && CMP == 0))) {
     // a compact variant whose plan equals the plain one's (nothing to leave out) is the same shape
     constexpr int cmp =
         RowGeo<T, N, ROW_STEP, R, PE, CL, CMP>::SMEM != RowGeo<T, N, ROW_STEP, R, PE, CL, 0>::SMEM ? CMP : 0;
-    for (int i = 0; i < o.n_row_variants; ++i)
+    for (int i = 0; i < o.n_row_variants && !again; ++i)
       if (o.row_step[i].rows == R && o.row_step[i].pe == cmin(PE, N / 2) && o.row_step[i].cl == CL &&
           o.row_step[i].cmp == cmp)
         return;   // same shape
@@ -230,9 +231,9 @@ static void add_row_variant(SizeOps& o) {
 }
 
 template <typename T, int N, int PE>
-static void add_col_variant(SizeOps& o) {
+static void add_col_variant(SizeOps& o, bool again = false) {
   if constexpr (ColGeo<T, N, COL_STEP, PE>::VALID && (N >= 64 || PE == default_step_col_pe<T, N>())) {
-    for (int i = 0; i < o.n_col_variants; ++i)
+    for (int i = 0; i < o.n_col_variants && !again; ++i)
       if (o.col_step[i].pe == cmin(PE, N)) return;
     StepVariant v{&launch_col_mode<T, N, COL_STEP, PE>, nullptr, nullptr, 1, cmin(PE, N), 1, 0};
     if constexpr (N <= kMaxBatchN) {
@@ -284,6 +285,13 @@ static SizeOps make_ops() {
     add_col_variant<T, N, 16>(o);
     add_col_variant<T, N, 4>(o);
   } else {
+    // Up to 256^2 the default is one of the other shapes; those keep the indices by which saved plans
+    // name them (rows 1: one row, 8 points; 2: one row, 4 points; columns 1: 4 points).
+    if constexpr (N >= 64 && N <= 256) {
+      add_row_variant<T, N, 1, 8>(o, true);
+      add_row_variant<T, N, 1, 4>(o, true);
+      add_col_variant<T, N, 4>(o, true);
+    }
     add_row_variant<T, N, 2, 8>(o);
     add_row_variant<T, N, 1, 8>(o);
     add_row_variant<T, N, 1, 4>(o);
