@@ -207,7 +207,7 @@ ttsh_status ttsh_time_kernels(ttsh_domain* d, int32_t iters, double* ms);
 /* Step-kernel tile shapes ("plan").  Each grid size has a list of row-pass variants (rows
  * per block, points per thread of the register butterflies) and column-pass variants
  * (points per thread); a domain starts with the entry measured
- * fastest for its size (entry 0 where batches take that size).  Variants compute the same step with a
+ * fastest for its size, entry 0 on grids up to 512^2.  Variants compute the same step with a
  * different factorisation of the transforms, so results agree to rounding, not bit for bit.
  * ttsh_autotune times every variant (as ttsh_time_kernels does, `iters` launches each, state
  * restored) and selects the fastest row and column variant.  plan (10 int32, may be NULL):
@@ -220,8 +220,9 @@ ttsh_status ttsh_time_kernels(ttsh_domain* d, int32_t iters, double* ms);
  * fit per SM and one block's staging and stores overlap the other's transforms.  ttsh_set_plan
  * selects variants by index (TTSH_E_INVALID if out of range).  ttsh_autotune times each row
  * variant with its G tile staged both ways where it can be (see ttsh_set_launch_mode), keeps the fastest
- * (variant, staging) pair, and then times whole steps (graphs of up to 64 steps, state
- * restored) with and without programmatic dependent launch and keeps the faster. */
+ * (variant, staging) pair and sets the launch mode: bit 0 on grids up to 512^2; beyond, it times
+ * whole steps (graphs of up to 64 steps, state restored) with and without programmatic
+ * dependent launch and sets bit 0 if that is faster, else leaves the choice to the library. */
 ttsh_status ttsh_autotune(ttsh_domain* d, int32_t iters, int32_t* plan);
 ttsh_status ttsh_get_plan(ttsh_domain* d, int32_t* plan);
 ttsh_status ttsh_set_plan(ttsh_domain* d, int32_t row_variant, int32_t col_variant);
@@ -229,8 +230,10 @@ ttsh_status ttsh_set_plan(ttsh_domain* d, int32_t row_variant, int32_t col_varia
 /* Launch mode of the step kernels, a bit set:
  *   bit 0  programmatic dependent launches: a pass may start (copy its twiddle tables and
  *          mask rows) while the previous pass is still running and waits on the device
- *          (griddepcontrol.wait) before it reads anything that pass wrote; on grids up to 512^2
- *          the library launches its steps so whatever the bit;
+ *          (griddepcontrol.wait) before it reads anything that pass wrote; clear: every
+ *          launch is an ordinary one.  Until a mode is set the library chooses: such launches
+ *          on grids up to 512^2, and beyond for steps that are not replayed from a graph
+ *          (ttsh_get_plan then reports bit 0 as 0);
  *   bit 1  the row pass loads its G tile with the tensor-memory accelerator (one 2D tile load
  *          per field, completion on an mbarrier with a bounded wait) instead of cp.async,
  *          where the tile allows it (N <= 512, a row segment of R complex values a multiple

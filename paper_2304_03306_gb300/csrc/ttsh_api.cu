@@ -834,6 +834,19 @@ void drop_record_graph(ttsh_domain* d) {
   d->rec_len = 0;
 }
 
+// Launch mode of the step kernels; graphs of another one are dropped.
+void set_mode(ttsh_domain* d, int pdl, int tma) {
+  if (pdl == d->dev.pdl && tma == d->dev.use_tma) return;
+  if (d->graph) {
+    cudaGraphExecDestroy(d->graph);
+    d->graph = nullptr;
+    d->graph_len = 0;
+  }
+  drop_record_graph(d);
+  d->dev.pdl = pdl;
+  d->dev.use_tma = tma;
+}
+
 // Graph of rec_len = every * floor(kGraphLen / every) steps with a sample at every
 // `every`-th step, starting with one.
 ttsh_status build_record_graph(ttsh_domain* d) {
@@ -955,7 +968,7 @@ ttsh_status ttsh_create_domain(const uint8_t* mask, const ttsh_params* p, void* 
   v.n = p->n;
   v.rec = nullptr;
   v.recctl = nullptr;
-  v.pdl = 0;
+  v.pdl = ttsh::kPdlAuto;
   v.whole = 0;
   v.captured = 0;
   v.use_tma = 0;
@@ -1323,34 +1336,28 @@ ttsh_status ttsh_autotune(ttsh_domain* d, int32_t iters, int32_t* plan) {
   d->dev.use_tma = tma0;
   if ((st = restore_state(d)) != TTSH_OK) return st;
   if ((st = ttsh_set_plan(d, br, bc)) != TTSH_OK) return st;
-  // launch mode: whole steps (row then column pass) with and without programmatic
-  // dependent launch; keep the faster (up to 512^2 steps overlap in either mode)
-  double t_mode[2] = {0, 0};
-  if (d->n <= ttsh::kPdlMaxN) return (st = ttsh_set_launch_mode(d, btma << 1)) != TTSH_OK ? st : ttsh_get_plan(d, plan);
-  for (int pdl = 0; pdl < 2; ++pdl) {
-    if ((st = ttsh_set_launch_mode(d, pdl | (btma << 1))) != TTSH_OK) return st;
-    if ((st = save_state(d)) != TTSH_OK) return st;
-    if ((st = time_steps(d, iters, &t_mode[pdl])) != TTSH_OK) return st;
-    if ((st = restore_state(d)) != TTSH_OK) return st;
+  // launch mode: up to 512^2 overlapped; beyond, whole steps (row then column pass) in graphs with and
+  // without programmatic dependent launch, and where that is not faster the library's rule
+  // (steps launched one by one overlap all the same)
+  if (d->n > ttsh::kPdlMaxN) {
+    double t_mode[2] = {0, 0};
+    for (int pdl = 0; pdl < 2; ++pdl) {
+      set_mode(d, pdl, btma);
+      if ((st = save_state(d)) != TTSH_OK) return st;
+      if ((st = time_steps(d, iters, &t_mode[pdl])) != TTSH_OK) return st;
+      if ((st = restore_state(d)) != TTSH_OK) return st;
+    }
+    set_mode(d, t_mode[1] < t_mode[0] ? 1 : ttsh::kPdlAuto, btma);
+  } else {
+    set_mode(d, 1, btma);
   }
-  if ((st = ttsh_set_launch_mode(d, (t_mode[1] < t_mode[0] ? 1 : 0) | (btma << 1))) != TTSH_OK) return st;
   return ttsh_get_plan(d, plan);
 }
 
 ttsh_status ttsh_set_launch_mode(ttsh_domain* d, int32_t mode) {
   if (!d) return fail(TTSH_E_INVALID, "domain is NULL");
   if (mode < 0 || mode > 3) return fail(TTSH_E_INVALID, "launch mode must be in [0, 3]");
-  const int pdl = mode & 1, tma = (mode >> 1) & 1;
-  if (pdl != d->dev.pdl || tma != d->dev.use_tma) {
-    if (d->graph) {
-      cudaGraphExecDestroy(d->graph);
-      d->graph = nullptr;
-      d->graph_len = 0;
-    }
-    drop_record_graph(d);
-    d->dev.pdl = pdl;
-    d->dev.use_tma = tma;
-  }
+  set_mode(d, mode & 1, (mode >> 1) & 1);
   return TTSH_OK;
 }
 
@@ -1364,7 +1371,7 @@ ttsh_status ttsh_get_plan(ttsh_domain* d, int32_t* plan) {
     plan[4] = d->ops.col_step[d->cv].pe;
     plan[5] = d->ops.n_row_variants;
     plan[6] = d->ops.n_col_variants;
-    plan[7] = d->dev.pdl | (d->dev.use_tma << 1);
+    plan[7] = (d->dev.pdl == 1 ? 1 : 0) | (d->dev.use_tma << 1);
     plan[8] = d->ops.row_step[d->rv].cl;
     plan[9] = d->ops.row_step[d->rv].cmp;
   }

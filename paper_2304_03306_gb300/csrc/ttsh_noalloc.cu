@@ -150,6 +150,7 @@ extern "C" ttsh_status ttsh_step_noalloc(const ttsh_params* p, const void* K, vo
   d.dx = p->dx;
   d.dt = p->dt;
   d.n = p->n;
+  d.pdl = 1;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // rebuild the row-pass inputs from the caller's state, then step
   e = ops.alone_prologue(d, s);

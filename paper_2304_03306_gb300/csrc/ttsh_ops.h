@@ -37,7 +37,7 @@ struct DomainDev {
   double a, b, lam, gv, gw, dx, dt;
   double cx, cy;   // centre for the order parameter
   int n;
-  int pdl;         // launch the step kernels with programmatic dependent launch
+  int pdl;         // launch the step kernels with programmatic dependent launch: 0, 1, or kPdlAuto
   int whole;       // never do (kernel timing: each launch runs by itself)
   int captured;    // the launches are being recorded into one of the library's graphs
   int use_tma;     // let the row step kernel load its G tile with the TMA (where tma_ok)
@@ -77,7 +77,8 @@ struct StepVariant {
 };
 
 constexpr int kMaxBatchN = 1024;
-constexpr int kPdlMaxN = 512;   // grids up to here: captured steps overlap in any launch mode
+constexpr int kPdlAuto = -1;    // DomainDev::pdl while no launch mode is set: the library's rule (step_pdl)
+constexpr int kPdlMaxN = 512;   // grids up to here overlap in graphs too
 
 constexpr int kAloneMaxN = 512;   // largest grid of ttsh_step_noalloc
 

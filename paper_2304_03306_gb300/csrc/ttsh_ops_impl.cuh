@@ -41,14 +41,17 @@ static int launch_smem(int smem, int grid, bool pdl) {
   return pdl && grid <= sm_count() && smem < kSpreadSmem ? kSpreadSmem : smem;
 }
 
-// Step kernels use programmatic dependent launch where the launch mode asks for it, when they
-// are launched one by one, and in graphs on grids up to 512^2 (results are the same bits).  One
-// by one the overlap hides the gap between launches (us a step: 256^2 float 12.0 -> 7.8, 1024^2
-// 26.8 -> 23.4, 2048^2 87.2 -> 81.9); in a graph it saves 0.5 us of a small grid's pass (256^2
-// 8.47 -> 7.34 us a step, 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1) but costs at 1024^2
-// (22.7 -> 23.8) and does nothing beyond.
+// Step kernels use programmatic dependent launch as the launch mode says; while none is set, where it
+// pays (results are the same bits): when they are launched one by one, and in graphs on grids up
+// to 512^2.  One by one the overlap hides the gap between launches (us a step: 256^2 float 12.0 ->
+// 7.8, 1024^2 26.8 -> 23.4, 2048^2 87.2 -> 81.9); in a graph it saves 0.5 us of a small grid's pass
+// (256^2 8.47 -> 7.34 us a step, 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1) but costs at
+// 1024^2 (22.7 -> 23.8) and does nothing beyond.
 template <int N>
-static bool step_pdl(const DomainDev& d) { return !d.whole && (d.pdl || !d.captured || N <= kPdlMaxN); }
+static bool step_pdl(const DomainDev& d) {
+  if (d.whole) return false;
+  return d.pdl == kPdlAuto ? !d.captured || N <= kPdlMaxN : d.pdl != 0;
+}
 
 // Launch, optionally as a programmatic dependent launch (the kernel may start while the
 // previous kernel in the stream is still running; it waits (griddepcontrol.wait) before it
