@@ -283,9 +283,7 @@ ttsh_status time_steps(ttsh_domain* d, int iters, double* ms) {
   const int reps = (iters + per - 1) / per;
   TTSH_CUDA(cudaStreamSynchronize(d->stream), "timing warm-up");
   TTSH_CUDA(cudaStreamBeginCapture(d->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
-  d->dev.captured = 1;
   for (int i = 0; i < per && st == TTSH_OK; ++i) st = one_step(d, d->capture);
-  d->dev.captured = 0;
   cudaGraph_t g = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(d->capture, &g);
   if (st != TTSH_OK || e2 != cudaSuccess) {
@@ -343,9 +341,7 @@ ttsh_status build_graph(ttsh_domain* d) {
   // The capture runs on a private stream; replays are launched on the domain's stream.
   TTSH_CUDA(cudaStreamBeginCapture(d->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
   ttsh_status st = TTSH_OK;
-  d->dev.captured = 1;
   for (int i = 0; i < kGraphLen && st == TTSH_OK; ++i) st = one_step(d, d->capture);
-  d->dev.captured = 0;
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(d->capture, &g);
   if (st != TTSH_OK) {
@@ -853,10 +849,8 @@ ttsh_status build_record_graph(ttsh_domain* d) {
   const int len = d->rec_every * (kGraphLen / d->rec_every);
   TTSH_CUDA(cudaStreamBeginCapture(d->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
   ttsh_status st = TTSH_OK;
-  d->dev.captured = 1;
   for (int i = 0; i < len && st == TTSH_OK; ++i)
     st = (i % d->rec_every == 0) ? record_step(d, d->capture) : one_step(d, d->capture);
-  d->dev.captured = 0;
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(d->capture, &g);
   if (st != TTSH_OK) {
@@ -970,7 +964,6 @@ ttsh_status ttsh_create_domain(const uint8_t* mask, const ttsh_params* p, void* 
   v.recctl = nullptr;
   v.pdl = ttsh::kPdlAuto;
   v.whole = 0;
-  v.captured = 0;
   v.use_tma = 0;
   v.err = reinterpret_cast<int*>(base + d->lay.err);
   v.knaive = reinterpret_cast<unsigned char*>(base + d->lay.knaive);

@@ -39,7 +39,6 @@ struct DomainDev {
   int n;
   int pdl;         // launch the step kernels with programmatic dependent launch: 0, 1, or kPdlAuto
   int whole;       // never do (kernel timing: each launch runs by itself)
-  int captured;    // the launches are being recorded into one of the library's graphs
   int use_tma;     // let the row step kernel load its G tile with the TMA (where tma_ok)
   int* err;        // device status word (bounded waits that ran out)
   // G as a 2D tensor for the row pass's TMA loads, one map per row-block height R = 1, 2, 4

@@ -41,6 +41,15 @@ static int launch_smem(int smem, int grid, bool pdl) {
   return pdl && grid <= sm_count() && smem < kSpreadSmem ? kSpreadSmem : smem;
 }
 
+// Whether launches on this stream go into a graph - the library's own, a corrected rollout's or the
+// caller's: the stream is asked, so that no capture has to say so.
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();   // (the legacy stream beside another's capture: the launch itself reports it)
+  return false;
+}
+
 // Step kernels use programmatic dependent launch as the launch mode says; while none is set, where it
 // pays (results are the same bits): when they are launched one by one, and in graphs on grids up
 // to 512^2.  One by one the overlap hides the gap between launches (us a step: 256^2 float 12.0 ->
@@ -48,9 +57,9 @@ static int launch_smem(int smem, int grid, bool pdl) {
 // (256^2 8.47 -> 7.34 us a step, 512^2 10.99 -> 9.81, 512^2 double 95.7 -> 94.1) but costs at
 // 1024^2 (22.7 -> 23.8) and does nothing beyond.
 template <int N>
-static bool step_pdl(const DomainDev& d) {
+static bool step_pdl(const DomainDev& d, cudaStream_t s) {
   if (d.whole) return false;
-  return d.pdl == kPdlAuto ? !d.captured || N <= kPdlMaxN : d.pdl != 0;
+  return d.pdl == kPdlAuto ? N <= kPdlMaxN || !capturing(s) : d.pdl != 0;
 }
 
 // Launch, optionally as a programmatic dependent launch (the kernel may start while the
@@ -104,7 +113,7 @@ static cudaError_t launch_row_kind(const DomainDev& d, cudaStream_t s) {
       a.tma = 1;
     }
   }
-  const bool pdl = KIND == ROW_STEP && step_pdl<N>(d);
+  const bool pdl = KIND == ROW_STEP && step_pdl<N>(d, s);
   return launch_k(row_kernel<T, N, KIND, R, PE, CL, CMP>, N / R, Geo::NT, launch_smem(Geo::SMEM, N / R, pdl), s, pdl,
                   CL, a, tm);
 }
@@ -120,7 +129,7 @@ static cudaError_t launch_col_mode(const DomainDev& d, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   // a recorded step adds one block that finishes the time-series sample
   const int extra = (MODE == COL_STEP && d.rec != nullptr) ? 1 : 0;
-  const bool pdl = MODE == COL_STEP && step_pdl<N>(d);
+  const bool pdl = MODE == COL_STEP && step_pdl<N>(d, s);
   return launch_k(col_kernel<T, N, MODE, PE, LEAN>, Geo::H + extra, Geo::NT, launch_smem(Geo::SMEM, Geo::H + extra, pdl), s,
                   pdl, 1, make_args<T>(d));
 }

@@ -100,3 +100,15 @@ def test_overlapped_and_ordinary_launches_leave_the_same_bits(T, n, prec):
     for mode in (None, 1):
         got = run(mode)
         assert all(np.array_equal(x, y) for x, y in zip(ref, got)), mode
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+def test_captured_steps_of_a_large_grid_are_ordinary_launches(T, cu, prec):
+    """While no mode is set, steps beyond 512^2 overlap one by one and not in a graph, whoever
+    records it (a corrected rollout's period, a caller)."""
+    torch = pytest.importorskip("torch")
+    stream = torch.cuda.Stream()
+    d = domain(T, 1024, prec)
+    assert programmatic_edges(cu, d, stream) == (5, 0)
+    d.synchronize()
+    d.close()
