@@ -233,7 +233,10 @@ ttsh_status ttsh_set_plan(ttsh_domain* d, int32_t row_variant, int32_t col_varia
  *          (griddepcontrol.wait) before it reads anything that pass wrote; clear: every
  *          launch is an ordinary one.  Until a mode is set the library chooses: such launches
  *          on grids up to 512^2, and beyond for steps that are not replayed from a graph
- *          (ttsh_get_plan then reports bit 0 as 0);
+ *          (ttsh_get_plan then reports bit 0 as 0).  Passes of few blocks reserve shared memory
+ *          so that these spread over the SMs; domains on streams of their own still share
+ *          them, but for a float 512^2 domain whose bit 0 was set (by the caller or the
+ *          autotuner), which keeps the SMs it runs on to itself;
  *   bit 1  the row pass loads its G tile with the tensor-memory accelerator (one 2D tile load
  *          per field, completion on an mbarrier with a bounded wait) instead of cp.async,
  *          where the tile allows it (N <= 512, a row segment of R complex values a multiple

@@ -18,9 +18,7 @@ static cudaError_t set_smem(K kernel, int bytes, std::atomic<int>& done) {
   return e;
 }
 
-// Shared memory a programmatic dependent launch of at most one block per SM reserves per
-// block: more than half an SM's, so that blocks admitted early (while the previous pass
-// still runs) cannot pile up two per SM and leave other SMs idle when they start.
+// Shared memory that the widest reservation of spread_smem takes; every step kernel allows it.
 constexpr int kSpreadSmem = 116 * 1024;
 
 static int sm_count() {
@@ -35,10 +33,27 @@ static int sm_count() {
   return v;
 }
 
-// Dynamic shared memory of a step-pass launch: the pass's own, or kSpreadSmem for a
-// programmatic dependent launch of at most one block per SM.
-static int launch_smem(int smem, int grid, bool pdl) {
-  return pdl && grid <= sm_count() && smem < kSpreadSmem ? kSpreadSmem : smem;
+// Shared memory that a programmatic dependent launch of at most one block per SM reserves per block,
+// so that blocks admitted early (while the previous pass still runs) cannot pile up on the SMs
+// that are free first and leave others idle when they start.  More than half an SM's keeps
+// every other block off it, those of domains stepped on streams of their own among them, so it
+// is left to a float 512^2 domain that was asked or tuned to overlap (us a step: one domain 9.5
+// reserved, 10.2 without; eight domains 44.4 and 25.8 a step of all, ordinary launches 29.2).
+// Double takes what leaves room for a second block from 256^2 (256^2: one domain 35.1 and 46.4
+// without, eight 137.5 and 136.9; with half an SM's 35.1 and 143.8) and for two more below
+// (128^2: one domain 20.3 and 24.4, eight 37.5 and 42.3; half an SM's 20.6 and 73.2).  Float grids
+// below 512^2 gain nothing by it (256^2: one domain 7.2 either way, sixteen 14.8 without and 42.9
+// with half an SM's, where ordinary launches take 17.4).
+template <typename T, int N>
+static int spread_smem(const DomainDev& d) {
+  if (sizeof(T) == 8) return (N >= 256 ? 92 : 73) * 1024;
+  return N == 512 && d.pdl == 1 ? kSpreadSmem : 0;
+}
+
+// Dynamic shared memory of a step-pass launch: the pass's own, or `spread` for a launch of at most
+// one block per SM.
+static int launch_smem(int smem, int grid, int spread) {
+  return smem < spread && grid <= sm_count() ? spread : smem;
 }
 
 // Whether launches on this stream go into a graph - the library's own, a corrected rollout's or the
@@ -114,7 +129,7 @@ static cudaError_t launch_row_kind(const DomainDev& d, cudaStream_t s) {
     }
   }
   const bool pdl = KIND == ROW_STEP && step_pdl<N>(d, s);
-  return launch_k(row_kernel<T, N, KIND, R, PE, CL, CMP>, N / R, Geo::NT, launch_smem(Geo::SMEM, N / R, pdl), s, pdl,
+  return launch_k(row_kernel<T, N, KIND, R, PE, CL, CMP>, N / R, Geo::NT, launch_smem(Geo::SMEM, N / R, pdl ? spread_smem<T, N>(d) : 0), s, pdl,
                   CL, a, tm);
 }
 
@@ -130,7 +145,7 @@ static cudaError_t launch_col_mode(const DomainDev& d, cudaStream_t s) {
   // a recorded step adds one block that finishes the time-series sample
   const int extra = (MODE == COL_STEP && d.rec != nullptr) ? 1 : 0;
   const bool pdl = MODE == COL_STEP && step_pdl<N>(d, s);
-  return launch_k(col_kernel<T, N, MODE, PE, LEAN>, Geo::H + extra, Geo::NT, launch_smem(Geo::SMEM, Geo::H + extra, pdl), s,
+  return launch_k(col_kernel<T, N, MODE, PE, LEAN>, Geo::H + extra, Geo::NT, launch_smem(Geo::SMEM, Geo::H + extra, pdl ? spread_smem<T, N>(d) : 0), s,
                   pdl, 1, make_args<T>(d));
 }
 

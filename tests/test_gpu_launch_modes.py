@@ -26,6 +26,8 @@ def cu():
     lib.cuStreamEndCapture.argtypes = [P, ctypes.POINTER(P)]
     lib.cuGraphGetEdges_v2.argtypes = [P, P, P, P, S]
     lib.cuGraphDestroy.argtypes = [P]
+    lib.cuGraphGetNodes.argtypes = [P, P, S]
+    lib.cuGraphKernelNodeGetParams_v2.argtypes = [P, P]
     return lib
 
 
@@ -35,8 +37,8 @@ def domain(T, n, prec):
     return d
 
 
-def programmatic_edges(cu, d, stream, steps=3):
-    """(edges, programmatic edges) between the kernels of `steps` steps."""
+def capture(cu, d, stream, steps):
+    """Graph of the domain's next steps (the state does not move)."""
     d.set_stream(stream.cuda_stream)
     d.step(1)   # the kernels' attributes, before the capture
     d.synchronize()
@@ -44,6 +46,12 @@ def programmatic_edges(cu, d, stream, steps=3):
     assert cu.cuStreamBeginCapture_v2(stream.cuda_stream, 1) == 0   # this thread's calls
     d.step(steps)
     assert cu.cuStreamEndCapture(stream.cuda_stream, ctypes.byref(graph)) == 0
+    return graph
+
+
+def programmatic_edges(cu, d, stream, steps=3):
+    """(edges, programmatic edges) between the kernels of `steps` steps."""
+    graph = capture(cu, d, stream, steps)
     k = ctypes.c_size_t(0)
     assert cu.cuGraphGetEdges_v2(graph, None, None, None, ctypes.byref(k)) == 0
     a, b = (ctypes.c_void_p * k.value)(), (ctypes.c_void_p * k.value)()
@@ -110,5 +118,34 @@ def test_captured_steps_of_a_large_grid_are_ordinary_launches(T, cu, prec):
     stream = torch.cuda.Stream()
     d = domain(T, 1024, prec)
     assert programmatic_edges(cu, d, stream) == (5, 0)
+    d.synchronize()
+    d.close()
+
+
+class KernelParams(ctypes.Structure):   # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("shared", ctypes.c_uint), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("n", [16, 64, 128, 256, 512])
+def test_a_step_leaves_room_on_an_sm_for_another_domain(T, cu, n, prec):
+    """A pass of fewer blocks than SMs does not keep the blocks of domains on other streams off its
+    SMs: two blocks fit (228 KB; 1 KB is the runtime's, up to 1 KB static)."""
+    torch = pytest.importorskip("torch")
+    stream = torch.cuda.Stream()
+    d = domain(T, n, prec)
+    graph = capture(cu, d, stream, 1)
+    k = ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(k)) == 0 and k.value == 2
+    nodes = (ctypes.c_void_p * k.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(k)) == 0
+    for node in nodes:
+        q = KernelParams()
+        assert cu.cuGraphKernelNodeGetParams_v2(node, ctypes.byref(q)) == 0
+        if q.grid[0] <= 148:
+            assert 2 * (q.shared + 2048) <= 228 * 1024, (list(q.grid), q.shared)
+    cu.cuGraphDestroy(graph)
     d.synchronize()
     d.close()
