@@ -761,9 +761,15 @@ struct ttsh_batch {
 namespace {
 
 constexpr int kBatchGraphLen = 32;
-// Items a step from which the persistent stepper's lean form pays (us a step, per-launch and lean
-// form: 12 domains, 1292 items 19.9 and 23.8; 26 domains, 3418 items 30.9 and 32.7; 32 domains,
-// 4128 items 37.1 and 33.6; 48 domains, 6448 items 57.7 and 50.3)
+// Items a step from which the persistent stepper's lean form pays.  Below, a step is a few rounds of
+// items for the 760 resident blocks of the per-launch form, and waits for each item's chain of
+// phases; above, the items an SM holds at once decide.  It is their number that counts, not their
+// size: batches of one size cross near 2600 items at 64^2, 3200 at 128^2, 3500 at 256^2 and 4500
+// at 512^2, the 48-domain sweep's subsets near 3600 (us a step, per-launch and lean form: 64^2,
+// 2112 items 16.7 and 26.5, 4224 items 29.7 and 22.3; 128^2, 2860 items 21.5 and 25.0, 3900
+// items 29.7 and 24.7; 256^2, 3096 items 27.7 and 28.4, 4128 items 36.9 and 32.1; 512^2, 3465
+// items 34.7 and 44.2, 4620 items 44.4 and 44.3; sweep, 2708 items 26.1 and 34.0, 3610 items
+// 32.5 and 32.3, 6448 items 58.5 and 50.4).
 constexpr int kLeanItems = 3700;
 
 ttsh_status batch_group_steps(BatchGroup& g, int nsteps, cudaStream_t s) {
@@ -1311,6 +1317,7 @@ ttsh_status ttsh_autotune(ttsh_domain* d, int32_t iters, int32_t* plan) {
   {
     const Whole whole(d->dev);
     for (int i = 0; i < d->ops.n_row_variants; ++i) {
+      if (ttsh::listed_before(d->ops.row_step, i)) continue;   // a shape under its other index
       for (int tma = 0; tma < 1 + d->ops.row_step[i].tma; ++tma) {   // G tile by cp.async, then by TMA (where the tile allows)
         d->dev.use_tma = tma;
         double t;
@@ -1321,6 +1328,7 @@ ttsh_status ttsh_autotune(ttsh_domain* d, int32_t iters, int32_t* plan) {
     d->dev.use_tma = btma;
     best = 1e300;
     for (int i = 0; i < d->ops.n_col_variants; ++i) {
+      if (ttsh::listed_before(d->ops.col_step, i)) continue;
       double t;
       if ((st = time_launches(d, d->ops.col_step[i].fn, iters, &t)) != TTSH_OK) return st;
       if (t < best) { best = t; bc = i; }

@@ -75,6 +75,13 @@ struct StepVariant {
   int tma;   // 1: the row pass can stage its G tile by TMA (launch mode bit 1)
 };
 
+// Whether entry i of a list of variants is an earlier entry's shape.
+inline bool listed_before(const StepVariant* v, int i) {
+  for (int k = 0; k < i; ++k)
+    if (v[k].fn == v[i].fn) return true;
+  return false;
+}
+
 constexpr int kMaxBatchN = 1024;
 constexpr int kPdlAuto = -1;    // DomainDev::pdl while no launch mode is set: the library's rule (step_pdl)
 constexpr int kPdlMaxN = 512;   // grids up to here overlap in graphs too
@@ -88,7 +95,7 @@ struct SizeOps {
   ColFn col;
   SpecFn spec;
   BlocksFn row_blocks;   // grid size of a row kernel kind (number of diagnostic partials)
-  int n_row_variants, n_col_variants;           // entry 0: the batches' tile shape
+  int n_row_variants, n_col_variants;           // entry 0: the default (see start_row for what a domain takes)
   StepVariant row_step[kMaxVariants];
   StepVariant col_step[kMaxVariants];
   int start_row, start_col;   // variants a domain starts with

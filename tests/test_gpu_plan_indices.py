@@ -41,3 +41,13 @@ def test_double_indices(T, n):
         points.add(d.plan()["col_points_per_thread"])
     assert shapes == {(2, 8), (1, 8), (1, 4)} and points == {8, 4}
     d.close()
+
+
+@pytest.mark.parametrize("n", [64, 128])
+def test_autotuner_names_a_shape_by_its_first_index(T, n):
+    """A tuned domain of the default shape keeps entry 0, with which a batch steps persistently."""
+    for _ in range(4):
+        d = T.Domain(np.zeros((n, n), np.uint8), n, 20.48 / n, precision=64)
+        plan = d.autotune(iters=4)
+        assert plan["row_variant"] != 2 and plan["col_variant"] != 1, plan
+        d.close()
