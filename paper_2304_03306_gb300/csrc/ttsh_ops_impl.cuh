@@ -41,13 +41,14 @@ static int sm_count() {
 // reserved, 10.2 without; eight domains 44.4 and 25.8 a step of all, ordinary launches 29.2).
 // Double takes what leaves room for a second block from 256^2 (256^2: one domain 35.1 and 46.4
 // without, eight 137.5 and 136.9; with half an SM's 35.1 and 143.8) and for two more below
-// (128^2: one domain 20.3 and 24.4, eight 37.5 and 42.3; half an SM's 20.6 and 73.2).  Float grids
-// below 512^2 gain nothing by it (256^2: one domain 7.2 either way, sixteen 14.8 without and 42.9
-// with half an SM's, where ordinary launches take 17.4).
+// (128^2: one domain 20.3 and 24.4, eight 37.5 and 42.3; half an SM's 20.6 and 73.2).  Float up to
+// 128^2 takes a quarter of an SM's (64^2: one domain 6.06 and 6.09, thirty-two 14.8 and 15.2; half
+// an SM's 6.06 and 19.3); at 256^2 it gains nothing (one domain 7.2 either way, sixteen 14.8
+// without and 42.9 with half an SM's, where ordinary launches take 17.4).
 template <typename T, int N>
 static int spread_smem(const DomainDev& d) {
   if (sizeof(T) == 8) return (N >= 256 ? 92 : 73) * 1024;
-  return N == 512 && d.pdl == 1 ? kSpreadSmem : 0;
+  return N <= 128 ? 54 * 1024 : N == 512 && d.pdl == 1 ? kSpreadSmem : 0;
 }
 
 // Dynamic shared memory of a step-pass launch: the pass's own, or `spread` for a launch of at most
